@@ -1,12 +1,12 @@
 // gs_fft.cuh -- register/shared-memory FFT building blocks for sm_103a.
 //
 // A length-n transform (n = 2^logn, 32 <= n <= 4096) is computed by a group
-// of T = n/32 threads; thread t holds the 32 elements x[t + T*i], i = 0..31,
-// in registers. The transform is a Stockham auto-sort FFT: a first radix-32
-// stage entirely in registers, then further stages of radix 32 (and one final
-// stage of radix 2..16 when log2(n) is not a multiple of 5), each preceded by
-// one exchange through the group's padded shared-memory buffer. The output is
-// left in registers in the same layout, in natural order.
+// of T = n/32 lanes, each of one or two threads; lane t holds the 32 elements
+// x[t + T*i], i = 0..31, in registers. The transform is a Stockham auto-sort
+// FFT: a first radix-32 stage in registers, then further stages of radix 32
+// (and one final stage of radix 2..16 when log2(n) is not a multiple of 5),
+// each preceded by one exchange through the group's padded shared-memory
+// buffer. The output is left in registers in the same layout, in natural order.
 //
 // Only the forward transform (kernel exp(-2 pi i jk/n), unnormalised) is
 // implemented. The inverse is obtained from it by exchanging real and
@@ -21,10 +21,20 @@ namespace gsk {
 
 __host__ __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-// a * w for a twiddle w = (c, s) meaning c + i s.
+// a * w for a twiddle w = (c, s) meaning c + i s. The fused operations are
+// written out here and in norm2: left to the compiler, the choice of the
+// product that is fused depends on the code around it, and the same
+// transform would round differently from kernel to kernel. (cmul_late: the
+// stage after 1024 points, which fuses the other product of the imaginary
+// part.)
 __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 w) {
-  return make_float2(a.x * w.x - a.y * w.y, a.x * w.y + a.y * w.x);
+  return make_float2(fmaf(a.x, w.x, -(a.y * w.y)), fmaf(a.y, w.x, a.x * w.y));
 }
+__device__ __forceinline__ float2 cmul_late(float2 a, float2 w) {
+  return make_float2(fmaf(a.x, w.x, -(a.y * w.y)), fmaf(a.x, w.y, a.y * w.x));
+}
+// x^2 + y^2
+__device__ __forceinline__ float norm2(float x, float y) { return fmaf(x, x, y * y); }
 
 // cos(2 pi e / 32) for e = 0..8, rounded to float.
 struct Cos32 {
@@ -46,41 +56,58 @@ struct W32 {
   static constexpr float S = (E <= 8) ? Cos32::v[8 - E] : Cos32::v[E - 8];
 };
 
+// Pairs of FP32 operations on the two halves of a float2, each rounded as the
+// scalar operation. On the device one instruction works on both halves: the
+// FP32 rate is the same (128 lanes per cycle and SM, measured for add,
+// multiply and fused multiply-add), but it takes half the issue slots and half
+// the code, and the kernels are bound by latency and instruction fetch rather
+// than by the FP32 pipe (64 mixed masks 15.38 -> 15.05 ms, 4 x 512^2 0.516 ->
+// 0.500 ms, 200 Adam steps at 1024^2 4.50 -> 4.37 ms).
+__host__ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+  return __ffma2_rn(a, b, c);
+#else
+  return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
+#endif
+}
+__host__ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
+#if defined(__CUDA_ARCH__) && __CUDA_ARCH__ >= 1000
+  return __fadd2_rn(a, b);
+#else
+  return cadd(a, b);
+#endif
+}
+
 // Radix-2 decimation-in-time butterfly (a, b) -> (a + w b, a - w b) with
 // w = W_32^E (0 <= E < 16). Trivial factors (1, -i) cost only additions,
 // (+-1 - i)/sqrt2 one addition pair less than a general factor, and the
 // general case uses fused multiply-adds with a - w b = 2a - (a + w b).
 template <int E>
 __host__ __device__ __forceinline__ void bfly(float2& a, float2& b) {
+  float2 s;
   if constexpr (E == 0) {
-    const float2 s = make_float2(a.x + b.x, a.y + b.y);
-    b = make_float2(a.x - b.x, a.y - b.y);
-    a = s;
+    s = add2(a, b);
+    b = fma2(b, make_float2(-1.f, -1.f), a);  // a - b, one rounding
   } else if constexpr (E == 8) {  // w = -i: w b = (b.y, -b.x)
-    const float2 s = make_float2(a.x + b.y, a.y - b.x);
+    s = make_float2(a.x + b.y, a.y - b.x);
     b = make_float2(a.x - b.y, a.y + b.x);
-    a = s;
   } else if constexpr (E == 4 || E == 12) {
     constexpr float c = Cos32::v[4];
     const float t1 = b.x + b.y;
     const float t2 = b.y - b.x;
-    if constexpr (E == 4) {  // w b = c t1 + i c t2
-      const float2 s = make_float2(fmaf(c, t1, a.x), fmaf(c, t2, a.y));
-      b = make_float2(fmaf(-c, t1, a.x), fmaf(-c, t2, a.y));
-      a = s;
-    } else {  // w b = c t2 - i c t1
-      const float2 s = make_float2(fmaf(c, t2, a.x), fmaf(-c, t1, a.y));
-      b = make_float2(fmaf(-c, t2, a.x), fmaf(c, t1, a.y));
-      a = s;
-    }
+    // w b = c t1 + i c t2 (E = 4), c t2 - i c t1 (E = 12)
+    const float2 u = E == 4 ? make_float2(t1, t2) : make_float2(t2, t1);
+    constexpr float cy = E == 4 ? c : -c;
+    s = fma2(make_float2(c, cy), u, a);
+    b = fma2(make_float2(-c, -cy), u, a);
   } else {
     constexpr float C = W32<E>::C;
     constexpr float S = W32<E>::S;
     // w b = (C b.x + S b.y) + i (C b.y - S b.x)
-    const float2 s = make_float2(fmaf(C, b.x, fmaf(S, b.y, a.x)), fmaf(C, b.y, fmaf(-S, b.x, a.y)));
-    b = make_float2(fmaf(2.f, a.x, -s.x), fmaf(2.f, a.y, -s.y));
-    a = s;
+    s = fma2(make_float2(C, C), b, fma2(make_float2(S, -S), make_float2(b.y, b.x), a));
+    b = fma2(make_float2(2.f, 2.f), a, make_float2(-s.x, -s.y));
   }
+  a = s;
 }
 
 // One decimation-in-time stage with half-span H on an R-array (bit-reversed
@@ -141,27 +168,63 @@ __host__ __device__ __forceinline__ void dft(float2 (&a)[R]) {
   for (int i = 0; i < R; ++i) a[i] = t[i];
 }
 
-// Per-group state of a distributed transform of length N = 2^LOGN by
-// T = N/32 threads. The geometry is a compile-time constant so that every
-// register and shared-memory index folds to an immediate offset.
-template <int LOGN>
+// Per-group state of a distributed transform of length N = 2^LOGN. The
+// geometry is a compile-time constant so that every register and
+// shared-memory index folds to an immediate offset.
+//
+// The line is laid out over T = N/32 lanes; lane t owns the 32 elements
+// x[t + T i'], i' = 0..31. S = 1: one thread holds all of them. S = 2: two
+// threads share a lane, thread c = 0, 1 with the 16 elements of parity
+// i' = 2 i + c; the two sit in the same lane of two neighbouring warps, so
+// that c is uniform over a warp. The transform evaluates the same butterflies
+// on the same operands in either form (the results are equal bit for bit):
+// the radix-2 decimation-in-time stages of a 32-point DFT work on the even and
+// the odd inputs separately until the last one, which pairs the two threads.
+//
+// Why S = 2: a lane's two transforms, projection and copies are a chain of
+// some 2600 dependent-issue instructions, which one warp alone on its
+// scheduler runs at 3.3 cycles each (4.1 us of a 5.4 us pass at 256 x 256,
+// 5.8-6.8 of 7-8 us at 1024 x 1024 where a scheduler has two such warps).
+// Two threads per lane halve the chain and double the warps in flight; the
+// price is one more exchange of half the line per 32-point DFT.
+template <int LOGN, int S = 1>
 struct GroupT {
   static constexpr int N = 1 << LOGN;
-  static constexpr int T = N >> 5;
+  static constexpr int T = N >> 5;         // lanes of a line
+  static constexpr int V = 32 / S;         // elements per thread
   static constexpr int SMEM = N + N / 32;  // padded exchange buffer (complex)
-  int t;                                   // thread index in the group, 0..T-1
-  int bar_id;                              // named barrier id (T > 32)
-  float2* sm;                              // this group's exchange buffer
+  static constexpr int TT = T > 32 ? T : 32;  // lanes that synchronise together (a team)
+  static constexpr int SPLIT = 16 * TT;    // a team's split-exchange buffer (complex), S = 2
+  static_assert(S == 1 || S == 2, "one or two threads per lane");
+  int t;                                   // lane in the line, 0..T-1
+  int c;                                   // parity of this thread's elements (0 if S = 1)
+  int bar_id;                              // named barrier id (S = 1: T > 32; S = 2: the team's)
+  float2* sm;                              // this line's exchange buffer
+  float2* sx;                              // the team's split-exchange buffer at this lane, S = 2
   const float2* __restrict__ tw;           // stage twiddle tables (twiddle_offset)
 
   __device__ __forceinline__ void sync() const {
-    if constexpr (T <= 32) {
+    if constexpr (S == 1 && T <= 32) {
       __syncwarp();
     } else {
-      asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(T) : "memory");
+      asm volatile("bar.sync %0, %1;" ::"r"(bar_id), "n"(S == 1 ? T : S * TT) : "memory");
     }
   }
+  // element index of register i is first() + STEP i
+  static constexpr int STEP = T * S;
+  __device__ __forceinline__ int first() const { return t + T * c; }
 };
+
+// This thread's lane of the block, and which of the lane's S threads it is:
+// the threads of a lane sit in neighbouring warps.
+template <int S>
+__device__ __forceinline__ int lane_of() {
+  return S == 1 ? threadIdx.x : ((threadIdx.x >> 6) << 5) | (threadIdx.x & 31);
+}
+template <int S>
+__device__ __forceinline__ int lane_part() {
+  return S == 1 ? 0 : (threadIdx.x >> 5) & 1;
+}
 
 // Twiddle tables. For the stage with Ns = 2^NSL and radix R the factors
 // W_{Ns R}^{r m} (1 <= m < R, r < Ns) are stored transposed, entry
@@ -171,104 +234,170 @@ struct GroupT {
 __host__ __device__ constexpr int twiddle_offset(int nsl) { return nsl == 5 ? 0 : 31 * 32; }
 
 // Twiddles of the stage that follows the first 32 points (NSL = 5), held in
-// registers: thread t needs W_{32 R}^{r m} for r = (t + T b) mod 32, b < 32/R,
-// 1 <= m < R. Loaded once and reused by every transform of the same length.
-template <int LOGN>
+// registers: the element i' = b + Q m of a lane (b < Q = 32/R) is multiplied
+// by W_{32 R}^{r m}, r = (t + T b) mod 32. Register i holds the factor of
+// element i' = S i + c; elements with m = 0 have none. Loaded once and reused
+// by every transform of the same length.
+template <int LOGN, int S = 1>
 struct StageTw {
   static constexpr int R = (LOGN <= 5) ? 1 : ((LOGN - 5 >= 5) ? 32 : (1 << (LOGN - 5)));
   static constexpr int Q = 32 / R;
-  static constexpr int COUNT = (R > 1) ? (R - 1) * Q : 1;
+  static constexpr int V = 32 / S;
+  static constexpr int COUNT = (R > 1) ? V : 1;
   float2 w[COUNT];
 
-  __device__ __forceinline__ void load(const float2* __restrict__ tw, int t) {
+  __device__ __forceinline__ void load(const float2* __restrict__ tw, int t, int c = 0) {
     if constexpr (R > 1) {
       constexpr int T = (1 << LOGN) >> 5;
 #pragma unroll
-      for (int b = 0; b < Q; ++b) {
+      for (int i = 0; i < V; ++i) {
+        const int ip = S * i + (S > 1 ? c : 0);
+        const int b = ip % Q, m = ip / Q;
         const int r = (t + T * b) & 31;
-#pragma unroll
-        for (int m = 1; m < R; ++m) w[b * (R - 1) + m - 1] = __ldg(tw + (m - 1) * 32 + r);
+        w[i] = m > 0 ? __ldg(tw + (m - 1) * 32 + r) : make_float2(1.f, 0.f);
       }
     }
   }
 };
 
-// Stockham stage of radix R with Ns = 2^NSL: butterflies j = t + T*b,
-// b < 32/R. Butterfly j reads x[j + m N/R] = v[b + (32/R) m], multiplies by
-// W_{Ns R}^{(j mod Ns) m} and transforms over m; for the last stage the
-// outputs land at the same register positions.
-template <int LOGN, int NSL, int R>
-__device__ __forceinline__ void stage_c(float2 (&v)[32], const GroupT<LOGN>& g, const StageTw<LOGN>& sw) {
+// The last radix-2 stage (half-span 16) of a 32-point DFT shared by the two
+// threads of a lane (S = 2): v holds the 16-point DFT of the thread's own
+// inputs, position k = 0..15. The thread of parity c forms the outputs k and
+// k + 16 of the positions k of its parity, which gives back the layout
+// i' = 2 i + c: it sends the positions of the other parity to its partner.
+template <int C, int K>
+__device__ __forceinline__ void split_bfly(float2 (&v)[16], float2 (&o)[16], const float2 (&r)[8]) {
+  if constexpr (K < 16) {
+    float2 a = C == 0 ? v[K] : r[K >> 1];
+    float2 b = C == 0 ? r[K >> 1] : v[K];
+    bfly<K>(a, b);
+    o[K >> 1] = a;
+    o[(K >> 1) + 8] = b;
+    split_bfly<C, K + 2>(v, o, r);
+  }
+}
+
+template <int C, class G>
+__device__ __forceinline__ void split_last(float2 (&v)[16], const G& g) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) g.sx[(2 * k + 1 - C) * G::TT] = v[2 * k + 1 - C];
+  g.sync();
+  float2 r[8], o[16];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) r[k] = g.sx[(2 * k + C) * G::TT];
+  split_bfly<C, C>(v, o, r);
+#pragma unroll
+  for (int i = 0; i < 16; ++i) v[i] = o[i];
+}
+
+// 32-point DFT over the elements i' of a lane.
+template <class G>
+__device__ __forceinline__ void dft32(float2 (&v)[G::V], const G& g) {
+  dft<G::V>(v);
+  if constexpr (G::V == 16) {
+    if (g.c == 0) split_last<0>(v, g);
+    else split_last<1>(v, g);
+  }
+}
+
+// Stockham stage of radix R with Ns = 2^NSL: butterflies j = t + T b,
+// b < Q = 32/R. Butterfly j reads x[j + m N/R], which is element i' = b + Q m,
+// multiplies by W_{Ns R}^{(j mod Ns) m} and transforms over m; the outputs
+// land at the same elements.
+template <int LOGN, int NSL, int R, int S>
+__device__ __forceinline__ void stage_c(float2 (&v)[32 / S], const GroupT<LOGN, S>& g, const StageTw<LOGN, S>& sw) {
   constexpr int Q = 32 / R;
   constexpr int T = GroupT<LOGN>::T;
   constexpr int NS = 1 << NSL;
+  // the threads of a lane share a radix-32 butterfly (parities of m); smaller
+  // ones stay within a thread (b = S q + c)
+  constexpr int QT = Q > S ? Q / S : 1;  // butterflies of this thread
+  constexpr int RT = R * Q / (S * QT);   // elements of each
 #pragma unroll
-  for (int b = 0; b < Q; ++b) {
-    float2 a[R];
+  for (int q = 0; q < QT; ++q) {
+    float2 a[RT];
 #pragma unroll
-    for (int m = 0; m < R; ++m) a[m] = v[b + Q * m];
+    for (int m = 0; m < RT; ++m) a[m] = v[q + QT * m];
     if constexpr (NSL == 5) {
+      if (S > 1 && Q == 1 && g.c != 0) a[0] = cmul(a[0], sw.w[0]);  // m = 1 here
 #pragma unroll
-      for (int m = 1; m < R; ++m) a[m] = cmul(a[m], sw.w[b * (R - 1) + m - 1]);
+      for (int m = 1; m < RT; ++m) a[m] = cmul(a[m], sw.w[q + QT * m]);
     } else if constexpr (NSL > 0) {
-      const int r = (g.t + T * b) & (NS - 1);
+      static_assert(NSL == 0 || R < 32, "lengths up to 4096 end their second radix-32 stage at 1024");
+      const int r = (g.t + T * (S * q + (S > 1 ? g.c : 0))) & (NS - 1);
       const float2* __restrict__ w = g.tw + twiddle_offset(NSL) + r;
 #pragma unroll
-      for (int m = 1; m < R; ++m) a[m] = cmul(a[m], __ldg(w + (m - 1) * NS));
+      for (int m = 1; m < R; ++m) a[m] = cmul_late(a[m], __ldg(w + (m - 1) * NS));
     }
-    dft<R>(a);
+    if constexpr (R == 32) dft32(a, g);
+    else dft<R>(a);
 #pragma unroll
-    for (int m = 0; m < R; ++m) v[b + Q * m] = a[m];
+    for (int m = 0; m < RT; ++m) v[q + QT * m] = a[m];
   }
 }
 
 // Exchange after a radix-32 stage with Ns = 2^NSL (butterfly j = t): output
 // m goes to (t / Ns) 32 Ns + (t mod Ns) + m Ns; then every thread reads back
-// x[t + T i]. Index i of the padded buffer lives at i + i/32.
-template <int LOGN, int NSL>
-__device__ __forceinline__ void exchange(float2 (&v)[32], const GroupT<LOGN>& g) {
+// its elements x[t + T i']. Index i of the padded buffer lives at i + i/32.
+//
+// S = 2 needs no second barrier: the buffer is next written behind the
+// barrier of the next split exchange, which every thread reaches after its
+// reads here.
+template <int LOGN, int NSL, int S>
+__device__ __forceinline__ void exchange(float2 (&v)[32 / S], const GroupT<LOGN, S>& g) {
   constexpr int T = GroupT<LOGN>::T;
+  constexpr int V = 32 / S;
   static_assert(NSL == 0 || NSL >= 5, "exchanges follow radix-32 stages");
+  const int c = S > 1 ? g.c : 0;
   if constexpr (NSL == 0) {
-    float2* w = g.sm + 33 * g.t;
+    float2* w = g.sm + 33 * g.t + c;
 #pragma unroll
-    for (int m = 0; m < 32; ++m) w[m] = v[m];
+    for (int i = 0; i < V; ++i) w[S * i] = v[i];
   } else {
     const int base = ((g.t >> NSL) << (NSL + 5)) + (g.t & ((1 << NSL) - 1));
-    float2* w = g.sm + base + (base >> 5);
     constexpr int STR = (1 << NSL) + (1 << (NSL - 5));
+    float2* w = g.sm + base + (base >> 5) + c * STR;
 #pragma unroll
-    for (int m = 0; m < 32; ++m) w[m * STR] = v[m];
+    for (int i = 0; i < V; ++i) w[S * i * STR] = v[i];
   }
   g.sync();
   if constexpr (T >= 32) {
-    const float2* r = g.sm + g.t + (g.t >> 5);
+    const float2* r = g.sm + g.t + (g.t >> 5) + c * (T + T / 32);
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = r[i * (T + T / 32)];
-  } else {
+    for (int i = 0; i < V; ++i) v[i] = r[S * i * (T + T / 32)];
+  } else if constexpr (S == 1) {
     const float2* r = g.sm + g.t;
 #pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = r[i * T + ((i * T) >> 5)];
+    for (int i = 0; i < V; ++i) v[i] = r[i * T + ((i * T) >> 5)];
+  } else {
+    // (2 i T + c T + t) >> 5 = (2 i T) >> 5: c T + t < 2 T divides 32
+    const float2* r = g.sm + g.t + c * T;
+#pragma unroll
+    for (int i = 0; i < V; ++i) v[i] = r[2 * i * T + ((2 * i * T) >> 5)];
   }
-  g.sync();
+  if constexpr (S == 1) g.sync();
 }
 
-template <int LOGN, int DONE>
-__device__ __forceinline__ void fft_from(float2 (&v)[32], const GroupT<LOGN>& g, const StageTw<LOGN>& sw) {
+template <int LOGN, int DONE, int S>
+__device__ __forceinline__ void fft_from(float2 (&v)[32 / S], const GroupT<LOGN, S>& g, const StageTw<LOGN, S>& sw) {
   if constexpr (DONE < LOGN) {
-    if constexpr (DONE > 0) exchange<LOGN, DONE - 5>(v, g);
+    if constexpr (DONE > 0) exchange<LOGN, DONE - 5, S>(v, g);
     constexpr int REM = LOGN - DONE;
     constexpr int RL = REM >= 5 ? 5 : REM;
-    stage_c<LOGN, DONE, (1 << RL)>(v, g, sw);
-    fft_from<LOGN, DONE + RL>(v, g, sw);
+    stage_c<LOGN, DONE, (1 << RL), S>(v, g, sw);
+    fft_from<LOGN, DONE + RL, S>(v, g, sw);
   }
 }
 
-// Forward unnormalised DFT of length N over the group: v holds x[t + T i] on
-// entry and X[t + T i] on exit. Every thread of the group must call it.
-template <int LOGN>
-__device__ __forceinline__ void group_fft(float2 (&v)[32], const GroupT<LOGN>& g, const StageTw<LOGN>& sw) {
-  fft_from<LOGN, 0>(v, g, sw);
+// Forward unnormalised DFT of length N over the group: the thread's registers
+// hold x[first() + STEP i] on entry and X[first() + STEP i] on exit. Every
+// thread of the team must call it. S = 2: other uses of the exchange buffer
+// after it start with a sync() (other threads may still be reading).
+template <int LOGN, int S>
+__device__ __forceinline__ void group_fft(float2 (&v)[32 / S], const GroupT<LOGN, S>& g, const StageTw<LOGN, S>& sw) {
+  // lengths that end in a 32-point DFT: its split exchange may still be read
+  if constexpr (S == 2 && LOGN % 5 == 0) g.sync();
+  fft_from<LOGN, 0, S>(v, g, sw);
 }
 
 }  // namespace gsk

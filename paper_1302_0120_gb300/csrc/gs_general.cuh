@@ -6,14 +6,17 @@
 // power-of-two kernel (gs_iterate.cuh); what differs is the transform and the
 // data movement:
 //   * The field B is stored row-major [ny][nx]; m transposed [nx][ny].
-//   * A row or column is transformed by a team of two warps (64 threads,
-//     four teams per block), which halves each transform's chain of
-//     dependent stage loops; teams synchronise on their own named barrier.
+//   * A row or column is transformed by a team of GenTeam::T threads; teams
+//     synchronise on their own named barrier. A block has as many teams as an
+//     SM has lines to do in one round (GenGeom, gs_internal.h): the passes are
+//     chains of dependent stage loops, and a second round costs a whole chain
+//     again (1280 x 1024 with four teams per block: 320 column groups on 256
+//     blocks, 35 us per column pass, of which the second round half).
 //   * A row pass gives each team one row: the row is read coalesced into the
 //     team's shared-memory buffer, transformed, projected and transformed
 //     again there, and written back coalesced.
-//   * A column pass moves 4 adjacent columns at a time: the block reads the
-//     [ny][4] tile in 32-byte row segments into four per-team column buffers,
+//   * A column pass moves one column per team at a time: the block reads the
+//     tile of adjacent columns in row segments into the teams' column buffers,
 //     each team transforms, projects and transforms its column, and the block
 //     writes the tile back the same way.
 //   * A length-n transform is a Stockham auto-sort FFT with radices 3 and 5
@@ -79,31 +82,49 @@ __host__ __device__ __forceinline__ void small_dft(float2 (&a)[R]) {
   else dft<R>(a);
 }
 
-// Barrier of team `team` (its two warps), named barrier 1 + team.
-__device__ __forceinline__ void team_sync(int team) {
-  asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kGenTeam) : "memory");
+// This thread's team and the team's size (a power of two of at least a warp).
+struct GenTeam {
+  int T;     // threads
+  int id;    // team in the block
+  int t;     // thread in the team
+  int n;     // teams of the block
+  __device__ explicit GenTeam(const Params& p)
+      : T(1 << p.gen_team_log), id(threadIdx.x >> p.gen_team_log), t(threadIdx.x & ((1 << p.gen_team_log) - 1)),
+        n(blockDim.x >> p.gen_team_log) {}
+  // named barrier 1 + id
+  __device__ __forceinline__ void sync() const {
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + id), "r"(T) : "memory");
+  }
+};
+
+// floor(a / b) for 0 <= a < 2^14, 0 < b < 2^14 through the reciprocal: (a + 1/2)/b
+// is at least 1/(2b) away from a whole number, further than its rounding
+// error. (Each stage of a transform needs four quotients and remainders by a
+// run-time length; the integer division sequence took longer than the stage.)
+__device__ __forceinline__ int small_div(int a, int b) {
+  return static_cast<int>((static_cast<float>(a) + 0.5f) * __fdividef(1.f, static_cast<float>(b)));
 }
 
 // One Stockham stage of radix R on a length-n transform whose first stages
 // formed sub-transforms of length ns: butterfly j = q ns + r reads
 // src[j + m n/R], multiplies by W_{ns R}^{r m} (stage table tw), transforms
 // over m and writes dst[q ns R + r + k ns]. Thread t of the team takes
-// butterflies t, t + 64, ...
+// butterflies t, t + T, ...
 template <int R>
 __device__ __forceinline__ void gen_stage(const float2* __restrict__ src, float2* __restrict__ dst, int n, int ns,
-                                          const float2* __restrict__ tw) {
+                                          const float2* __restrict__ tw, const GenTeam& tm) {
   constexpr int U = 1;
   const int nb = n / R;
-  const int tt = threadIdx.x % kGenTeam;
-  const int qinc = kGenTeam / ns, rinc = kGenTeam % ns;
-  int q = tt / ns, r = tt % ns;
+  const int tt = tm.t;
+  const int qinc = small_div(tm.T, ns), rinc = tm.T - qinc * ns;
+  int q = small_div(tt, ns), r = tt - q * ns;
   const float2* const tws = tw + (ns - 1);
-  for (int j0 = tt; j0 < nb; j0 += kGenTeam * U) {
+  for (int j0 = tt; j0 < nb; j0 += tm.T * U) {
     float2 a[U][R];
     int base[U], rr[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      const int j = j0 + kGenTeam * u;
+      const int j = j0 + tm.T * u;
       rr[u] = r;
       base[u] = q * ns * R + r;
       if (j < nb) {
@@ -120,14 +141,14 @@ __device__ __forceinline__ void gen_stage(const float2* __restrict__ src, float2
     if (ns > 1) {
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if (j0 + kGenTeam * u < nb) {
+        if (j0 + tm.T * u < nb) {
 #pragma unroll
           for (int m = 1; m < R; ++m) a[u][m] = cmul(a[u][m], tws[(m - 1) * ns + rr[u]]);
         }
     }
 #pragma unroll
     for (int u = 0; u < U; ++u)
-      if (j0 + kGenTeam * u < nb) {
+      if (j0 + tm.T * u < nb) {
         small_dft<R>(a[u]);
 #pragma unroll
         for (int k = 0; k < R; ++k) dst[base[u] + k * ns] = a[u][k];
@@ -135,23 +156,23 @@ __device__ __forceinline__ void gen_stage(const float2* __restrict__ src, float2
   }
 }
 
-// Forward unnormalised DFT of the length-n vector in `a` by team `team`,
+// Forward unnormalised DFT of the length-n vector in `a` by the team,
 // using `b` as the second buffer; returns the buffer that holds the result
 // (a for an even number of stages, b for an odd one).
 __device__ __forceinline__ float2* gen_fft(float2* a, float2* b, int n, unsigned plan, int nst, const float2* tw,
-                                           int team) {
+                                           const GenTeam& tm) {
   int ns = 1;
 #pragma unroll 1
   for (int s = 0; s < nst; ++s) {
     const int R = radix_of_code((plan >> (3 * s)) & 7u);
     switch (R) {
-      case 2: gen_stage<2>(a, b, n, ns, tw); break;
-      case 3: gen_stage<3>(a, b, n, ns, tw); break;
-      case 4: gen_stage<4>(a, b, n, ns, tw); break;
-      case 5: gen_stage<5>(a, b, n, ns, tw); break;
-      default: gen_stage<8>(a, b, n, ns, tw); break;
+      case 2: gen_stage<2>(a, b, n, ns, tw, tm); break;
+      case 3: gen_stage<3>(a, b, n, ns, tw, tm); break;
+      case 4: gen_stage<4>(a, b, n, ns, tw, tm); break;
+      case 5: gen_stage<5>(a, b, n, ns, tw, tm); break;
+      default: gen_stage<8>(a, b, n, ns, tw, tm); break;
     }
-    team_sync(team);
+    tm.sync();
     ns *= R;
     float2* t = a;
     a = b;
@@ -163,26 +184,36 @@ __device__ __forceinline__ float2* gen_fft(float2* a, float2* b, int n, unsigned
 // Copy the twiddle tables to shared memory (once per launch).
 __device__ __forceinline__ void gen_load_twiddles(const Params& p, unsigned char* smem) {
   float2* t = reinterpret_cast<float2*>(smem);
-  for (int e = threadIdx.x; e < p.nx; e += kThreads) t[e] = p.twx[e];
-  for (int e = threadIdx.x; e < p.ny; e += kThreads) t[p.nx + e] = p.twy[e];
+  for (int e = threadIdx.x; e < p.nx; e += blockDim.x) t[e] = p.twx[e];
+  for (int e = threadIdx.x; e < p.ny; e += blockDim.x) t[p.nx + e] = p.twy[e];
   __syncthreads();
 }
 
-// m = s sqrt(I), transposed ([nx][ny]), for this block's columns.
-__device__ __forceinline__ void gen_build_amplitude(const Params& p, int mb, float s) {
+// m = s sqrt(I), transposed ([nx][ny]), for this block's columns: tiles of 8
+// columns go through the (still unused) team buffers, so that both sides are
+// read and written in segments (lanes striding over rows took 20 us once per
+// run at 1280 x 1024).
+__device__ __forceinline__ void gen_build_amplitude(const Params& p, int mb, float s, unsigned char* smem) {
   const size_t moff = static_cast<size_t>(mb) * static_cast<size_t>(p.mstride);
   const float* const Im = p.I + moff;
   float* const mTm = p.mT + moff;
+  const int ny = p.ny;
+  float* const tile = reinterpret_cast<float*>(reinterpret_cast<float2*>(smem) + gen_tw_entries(p.nx, ny));
   const int lo = split(blockIdx.x, gridDim.x, p.nx);
   const int hi = split(blockIdx.x + 1, gridDim.x, p.nx);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int x = lo + w; x < hi; x += kThreads / 32)
-    for (int y = lane; y < p.ny; y += 32)
-      mTm[static_cast<size_t>(x) * p.ny + y] = s * sqrtf(Im[static_cast<size_t>(y) * p.nx + x]);
-  __syncthreads();
+  const int k = threadIdx.x & 7;
+  for (int c0 = lo; c0 < hi; c0 += 8) {
+    const int wc = min(8, hi - c0);
+    if (k < wc)
+      for (int y = threadIdx.x >> 3; y < ny; y += blockDim.x >> 3)
+        tile[k * (ny + 1) + y] = Im[static_cast<size_t>(y) * p.nx + c0 + k];
+    __syncthreads();
+    for (int c = 0; c < wc; ++c)
+      for (int y = threadIdx.x; y < ny; y += blockDim.x)
+        mTm[static_cast<size_t>(c0 + c) * ny + y] = s * sqrtf(tile[c * (ny + 1) + y]);
+    __syncthreads();
+  }
 }
-
-
 
 // Wrap an angle as the power-of-two kernel does: (-pi, pi].
 __device__ __forceinline__ float gen_phase(float2 u) {
@@ -190,7 +221,7 @@ __device__ __forceinline__ float gen_phase(float2 u) {
   return (a <= -3.14159274f) ? 3.14159274f : a;
 }
 
-// One pass over rows [lo, hi) (kInit, kRow) or 8-column groups [lo, hi)
+// One pass over rows [lo, hi) (kInit, kRow) or columns [lo, hi)
 // (kCol, kResid, kInitM) of mask mb. Returns this thread's FP64 contribution
 // to the pass's gap sum.
 static __device__ __forceinline__ float run_pass_gen(const Params& p, int mb, int kind, bool last, int lo, int hi,
@@ -203,25 +234,26 @@ static __device__ __forceinline__ float run_pass_gen(const Params& p, int mb, in
   const float2* twx = reinterpret_cast<const float2*>(smem);
   const float2* twy = twx + nx;
   float2* wbase = reinterpret_cast<float2*>(smem) + gen_tw_entries(nx, ny);
-  const int tm = threadIdx.x / kGenTeam, tt = threadIdx.x % kGenTeam;
-  float2* const A = wbase + tm * gen_team_stride(nmax);
+  const GenTeam tm(p);
+  const int tt = tm.t, T = tm.T;
+  float2* const A = wbase + tm.id * gen_team_stride(nmax);
   float2* const Bf = A + nmax + 1;
   const float inv_sqrt_n = p.inv_sqrt_n;
   const bool two = (kind == kCol || (kind == kRow && !(last && !p.final_resid)));
   float acc = 0.f;
 
   if (kind == kInit || kind == kRow) {
-    for (int row = lo + tm; row < hi; row += kGenTeams) {
+    for (int row = lo + tm.id; row < hi; row += tm.n) {
       float2* src = Bm + static_cast<size_t>(row) * nx;
       const float* pp = p.p_slm ? p.p_slm + static_cast<size_t>(row) * nx : nullptr;
       if (kind == kInit) {
         const float* ph = p.phi_in + moff + static_cast<size_t>(row) * nx;
         float* po = p.phi_out + moff + static_cast<size_t>(row) * nx;
-        for (int x0 = tt; x0 < nx; x0 += kGenTeam * 4) {
+        for (int x0 = tt; x0 < nx; x0 += T * 4) {
           float f[4], a[4];
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const int x = x0 + kGenTeam * k;
+            const int x = x0 + T * k;
             f[k] = x < nx ? ph[x] : 0.f;
             a[k] = (pp && x < nx) ? pp[x] : 1.f;  // u0 = p exp(i phi0)
           }
@@ -229,32 +261,32 @@ static __device__ __forceinline__ float run_pass_gen(const Params& p, int mb, in
           for (int k = 0; k < 4; ++k) {
             float s, c;
             sincosf(f[k], &s, &c);
-            if (x0 + kGenTeam * k < nx) A[x0 + kGenTeam * k] = make_float2(a[k] * c, a[k] * s);
+            if (x0 + T * k < nx) A[x0 + T * k] = make_float2(a[k] * c, a[k] * s);
           }
         }
         if (last) {  // zero iterations
-          team_sync(tm);
-          for (int x = tt; x < nx; x += kGenTeam) po[x] = gen_phase(A[x]);
+          tm.sync();
+          for (int x = tt; x < nx; x += T) po[x] = gen_phase(A[x]);
         }
       } else {
-        for (int x = tt; x < nx; x += kGenTeam) cp_async8(A + x, src + x);
+        for (int x = tt; x < nx; x += T) cp_async8(A + x, src + x);
         cp_async_wait_all();
       }
-      team_sync(tm);
+      tm.sync();
       float2* res = gen_fft(A, Bf, nx, p.planx, p.nstx, twx, tm);
       if (kind == kRow) {
         // res = swap(IDFT_x(B)) = swap(sqrt(N) P_M u^nu): gap to S, Eq. (e:PS)
         float part = 0.f;
-        for (int x0 = tt; x0 < nx; x0 += kGenTeam * 8) {
+        for (int x0 = tt; x0 < nx; x0 += T * 8) {
           float a[8];
 #pragma unroll
-          for (int k = 0; k < 8; ++k) a[k] = (pp && x0 + kGenTeam * k < nx) ? pp[x0 + kGenTeam * k] : 1.f;
+          for (int k = 0; k < 8; ++k) a[k] = (pp && x0 + T * k < nx) ? pp[x0 + T * k] : 1.f;
           float2 t8[8];
 #pragma unroll
-          for (int k = 0; k < 8; ++k) t8[k] = (x0 + kGenTeam * k < nx) ? res[x0 + kGenTeam * k] : make_float2(1.f, 0.f);
+          for (int k = 0; k < 8; ++k) t8[k] = (x0 + T * k < nx) ? res[x0 + T * k] : make_float2(1.f, 0.f);
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
-            const int x = x0 + kGenTeam * k;
+            const int x = x0 + T * k;
             if (x < nx) {
               const float2 t = t8[k];
               const float vx = t.y, vy = t.x;
@@ -269,60 +301,59 @@ static __device__ __forceinline__ float run_pass_gen(const Params& p, int mb, in
           }
         }
         acc += part;
-        team_sync(tm);
+        tm.sync();
         if (last) {
           float* po = p.phi_out + moff + static_cast<size_t>(row) * nx;
-          for (int x = tt; x < nx; x += kGenTeam) po[x] = gen_phase(res[x]);
+          for (int x = tt; x < nx; x += T) po[x] = gen_phase(res[x]);
         }
         if (two) res = gen_fft(res, res == A ? Bf : A, nx, p.planx, p.nstx, twx, tm);
       }
       if (kind == kInit || two)
-        for (int x = tt; x < nx; x += kGenTeam) src[x] = res[x];
-      team_sync(tm);
+        for (int x = tt; x < nx; x += T) src[x] = res[x];
+      tm.sync();
     }
     return acc;
   }
 
-  // Column passes: groups of 4 adjacent columns; team k owns column c0 + k.
+  // Column passes: groups of adjacent columns; team k owns column c0 + k.
   const int stride = gen_team_stride(nmax);
   const bool store = (kind == kCol || kind == kInitM);
   // which of a warp's buffers holds the stored result: A after two transforms,
   // else A or Bf by the parity of the stage count
   const int out_off = (kind == kCol || (p.nsty & 1) == 0) ? 0 : nmax + 1;
-  for (int cg = lo; cg < hi; ++cg) {
-    const int c0 = cg * kGenTeams;
-    const int wc = min(kGenTeams, nx - c0);
+  // the tile's copies: this thread's column of the group, and its first row
+  // and row step (T rows per sweep of the block)
+  const int cy = small_div(threadIdx.x, tm.n), ck = threadIdx.x - cy * tm.n;
+  for (int c0 = lo; c0 < hi; c0 += tm.n) {
+    const int wc = min(tm.n, hi - c0);
     __syncthreads();  // the previous group's tile has been written back
-    {
-      const int k = threadIdx.x % kGenTeams;  // column of this thread in every round
-      if (k < wc) {
-        if (kind == kInitM) {
-          for (int y = threadIdx.x / kGenTeams; y < ny; y += kThreads / kGenTeams)  // swap((m, 0))
-            wbase[k * stride + y] = make_float2(0.f, mTm[static_cast<size_t>(c0 + k) * ny + y]);
-        } else {
-          for (int y = threadIdx.x / kGenTeams; y < ny; y += kThreads / kGenTeams)
-            cp_async8(wbase + k * stride + y, Bm + static_cast<size_t>(y) * nx + c0 + k);
-          cp_async_wait_all();
-        }
+    if (ck < wc) {
+      float2* const col = wbase + ck * stride;
+      if (kind == kInitM) {
+        for (int y = cy; y < ny; y += T)  // swap((m, 0))
+          col[y] = make_float2(0.f, mTm[static_cast<size_t>(c0 + ck) * ny + y]);
+      } else {
+        for (int y = cy; y < ny; y += T) cp_async8(col + y, Bm + static_cast<size_t>(y) * nx + c0 + ck);
+        cp_async_wait_all();
       }
     }
     __syncthreads();
-    if (tm < wc) {
+    if (tm.id < wc) {
       float2* res = gen_fft(A, Bf, ny, p.plany, p.nsty, twy, tm);
       if (kind != kInitM) {
         // res = Y = F u^nu along this column: residual and Eq. (e:Mhat)
-        const float* mcol = mTm + static_cast<size_t>(c0 + tm) * ny;
+        const float* mcol = mTm + static_cast<size_t>(c0 + tm.id) * ny;
         float part = 0.f;
-        for (int y0 = tt; y0 < ny; y0 += kGenTeam * 8) {
+        for (int y0 = tt; y0 < ny; y0 += T * 8) {
           float mv[8];
           float2 yv[8];
 #pragma unroll
-          for (int u = 0; u < 8; ++u) mv[u] = (y0 + kGenTeam * u < ny) ? mcol[y0 + kGenTeam * u] : 0.f;
+          for (int u = 0; u < 8; ++u) mv[u] = (y0 + T * u < ny) ? mcol[y0 + T * u] : 0.f;
 #pragma unroll
-          for (int u = 0; u < 8; ++u) yv[u] = (y0 + kGenTeam * u < ny) ? res[y0 + kGenTeam * u] : make_float2(1.f, 0.f);
+          for (int u = 0; u < 8; ++u) yv[u] = (y0 + T * u < ny) ? res[y0 + T * u] : make_float2(1.f, 0.f);
 #pragma unroll
           for (int u = 0; u < 8; ++u) {
-            const int y = y0 + kGenTeam * u;
+            const int y = y0 + T * u;
             if (y < ny) {
               const float m = mv[u];
               const float2 Y = yv[u];
@@ -340,15 +371,15 @@ static __device__ __forceinline__ float run_pass_gen(const Params& p, int mb, in
           }
         }
         acc += part;
-        team_sync(tm);
+        tm.sync();
         if (kind == kCol) res = gen_fft(res, res == A ? Bf : A, ny, p.plany, p.nsty, twy, tm);
       }
     }
     if (store) {
       __syncthreads();
-      for (int e = threadIdx.x; e < ny * kGenTeams; e += kThreads) {
-        const int y = e / kGenTeams, k = e % kGenTeams;
-        if (k < wc) Bm[static_cast<size_t>(y) * nx + c0 + k] = wbase[k * stride + out_off + y];
+      if (ck < wc) {
+        const float2* const col = wbase + ck * stride + out_off;
+        for (int y = cy; y < ny; y += T) Bm[static_cast<size_t>(y) * nx + c0 + ck] = col[y];
       }
     }
   }

@@ -5,7 +5,14 @@
 
 namespace gsk {
 
-constexpr int kThreads = 256;                   // threads per block of the iteration kernel
+// A block of the iteration kernels works on 256 lanes of 32 values, each held
+// by one thread or by two (GroupT, gs_fft.cuh).
+constexpr int kThreads = 256;
+constexpr int kMaxThreads = 2 * kThreads;
+// Threads per lane of the FP32 kernel of an nx x ny grid of powers of two.
+inline __host__ __device__ constexpr int iteration_split(int nx, int ny) { return (nx > 512 || ny > 512) ? 1 : 2; }
+constexpr int kMixedSplit = 1;  // ... of the mixed and serving kernels
+constexpr int kLossSplit = 2;   // ... of the loss kernel
 constexpr int kMaxIterPerLaunch = 128;          // iterations per persistent launch
 constexpr int kSlots = 2 * kMaxIterPerLaunch + 2;  // FP64 partial-sum slots per launch
 constexpr int kMaxGrid = 256;                   // upper bound on blocks per launch
@@ -16,6 +23,12 @@ constexpr int kTraceRows = 2 * kMaxIterPerLaunch + 4;
 // Group exchange buffers: (256 / T) groups of (n + n/32) complex, T = n/32,
 // which is 256 * 33 complex whatever n is.
 constexpr int kGroupSmemBytes = kThreads * 33 * 8;
+// Split-exchange buffers of the kernels with two threads per lane: 16 complex
+// values per lane. The FP32 kernels with one thread per lane have a second
+// staging buffer for column blocks there.
+constexpr int kSplitSmemBytes = kThreads * 16 * 8;
+constexpr int kAheadSmemBytes = 8192 * 8;
+constexpr int lane_smem_bytes(int split) { return split > 1 ? kSplitSmemBytes : kAheadSmemBytes; }
 // Extra shared memory of the tensor-core kernels: stage twiddles [32][32]
 // complex and a 32-entry cos/sin table (mma.sync); the two DFT matrices (hi
 // and lo parts, 8 KiB each) and an 8 KiB twiddle table (tcgen05, whose
@@ -69,6 +82,7 @@ struct Params {
   // radix kRadixOf[c]), first stage in the low bits, and the stage counts.
   unsigned planx, plany;
   int nstx, nsty;
+  int gen_teams, gen_team_log;  // teams of a block, log2 of a team's threads
 };
 
 // Three size classes in one launch: square grids 256, 512 and 1024
@@ -113,19 +127,45 @@ inline __host__ __device__ bool uses_rg(int nx, int ny) {
 constexpr int kMaxGeneralSide = 1536;
 constexpr int kMaxGeneralStages = 10;
 
-// The general kernel transforms a row or column with a team of two warps;
-// a block holds four teams.
-constexpr int kGenTeam = 64;
-constexpr int kGenTeams = kThreads / kGenTeam;
+// The general kernel transforms a row or column with a team of threads; a
+// block has at most kGenMaxTeams teams, and one block runs per SM.
+constexpr int kGenMaxTeams = 10;
+constexpr int kGenMaxThreads = 640;
+static_assert(kGenMaxTeams << 6 <= kGenMaxThreads, "teams of two warps fit");
+constexpr int kGenSmemLimit = 227 * 1024 - 2048;  // dynamic part; the rest is the block's static arrays
 
 // Shared-memory layout of the general kernel: the two twiddle tables (nx,
 // then ny complex), then per team two buffers of max(nx, ny) complex.
 inline __host__ __device__ int gen_tw_entries(int nx, int ny) { return (nx + ny + 1) & ~1; }
 inline __host__ __device__ int gen_team_stride(int nmax) { return 2 * nmax + 2; }  // complex; 16-byte multiple
-inline __host__ __device__ size_t gen_smem_bytes(int nx, int ny) {
+inline __host__ __device__ size_t gen_smem_bytes(int nx, int ny, int teams) {
   const int nmax = nx > ny ? nx : ny;
-  return (static_cast<size_t>(gen_tw_entries(nx, ny)) + static_cast<size_t>(kGenTeams) * gen_team_stride(nmax)) *
+  return (static_cast<size_t>(gen_tw_entries(nx, ny)) + static_cast<size_t>(teams) * gen_team_stride(nmax)) *
          sizeof(float2);
+}
+
+// Teams per block and log2 of a team's threads for `masks` masks of nx x ny
+// on `sms` SMs: the fewest rounds that shared memory allows, then the fewest
+// teams that need no more (at least 4, so that column tiles are 32-byte row
+// segments).
+struct GenGeom {
+  int teams;
+  int team_log;
+};
+inline GenGeom gen_geom(int nx, int ny, int masks, int sms) {
+  const int nmax = nx > ny ? nx : ny;
+  int fit = kGenMaxTeams;
+  while (fit > 4 && gen_smem_bytes(nx, ny, fit) > static_cast<size_t>(kGenSmemLimit)) --fit;
+  const long long lines = static_cast<long long>(nmax) * masks;
+  const long long rounds = (lines + static_cast<long long>(sms) * fit - 1) / (static_cast<long long>(sms) * fit);
+  const long long per = static_cast<long long>(sms) * rounds;
+  int teams = static_cast<int>((lines + per - 1) / per);
+  if (teams < 4) teams = 4;
+  // two warps per line; four for the longer ones, where a block has room
+  // (640 x 480: 384 -> 374 us per 20 iterations; 120 x 90: 246 -> 272)
+  int tl = nmax >= 300 ? 7 : 6;
+  if ((teams << tl) > kGenMaxThreads) tl = 6;
+  return {teams, tl};
 }
 
 // Kernel for log2(nx) = LX and the given log2(ny); defined per LX in gs_inst.cu.

@@ -53,11 +53,29 @@ constexpr int kTcTwOffset = kBlockSmemOffset + kBlockSmemBytes;
 constexpr int kTcCsOffset = kTcTwOffset + kTcTwBytes;
 static_assert(kTcTwBytes + kTcCsBytes == kTcExtraSmemBytes, "tensor-core tables match the launch size");
 
-// Stands in for TcFft in the kernels whose transforms run on the FP32 ALUs.
+// Stands in for TcFft in the kernels whose transforms run on the FP32 ALUs,
+// S threads per lane; AHEAD: the kernel has the second staging buffer.
+template <int S, bool AHEAD = S == 1>
 struct NoTc {
+  static constexpr int kThreadsPerLane = S;
+  static constexpr bool kAhead = AHEAD;
   static constexpr bool kEnabled = false;
   static constexpr bool kTcgen05 = false;
 };
+
+// Column blocks of the next round are loaded during a round.
+template <class TCF>
+__host__ __device__ constexpr bool loads_ahead() {
+  if constexpr (TCF::kEnabled) return false;
+  else return TCF::kAhead;
+}
+
+// Threads per lane of a kernel whose transforms are TCF's.
+template <class TCF>
+__host__ __device__ constexpr int lane_threads() {
+  if constexpr (TCF::kEnabled) return 1;
+  else return TCF::kThreadsPerLane;
+}
 
 // Storage of the field B between passes: column blocks of W adjacent columns,
 // each block one contiguous [ny][W] array, with the W elements of each of its
@@ -65,31 +83,37 @@ struct NoTc {
 // bulk copy each way and reads its columns from shared memory without bank
 // conflicts; a row pass reads and writes 8W-byte row segments.
 //
-// P column blocks are in flight per round of a column pass: P = 2 when a
-// block of W = 8 columns fills only half of the thread block (512-point
-// columns). Each half (slot) then loads, transforms and stores its own column
-// block on its own mbarrier, so that all threads work and the copies of one
-// half overlap the transforms of the other. (Blocks of 4 columns for
+// P column blocks are in flight per round of a column pass: P = 2 (4) when a
+// block of W = 8 columns fills only a half (a quarter) of the thread block
+// (512-point, 256-point columns). Each slot of the threads then loads,
+// transforms and stores its own column block on its own mbarrier, so that all
+// threads work and the copies of one slot overlap the transforms of the
+// others. (Blocks of 4 columns for
 // 1024-point columns, two per round, were measured slower: the column pass
 // gained 0.26 us, but the row pass, now reading 32-byte segments from twice
-// as many lines, lost 0.5 us.) kPaired = false keeps one block per round (the
-// loss kernel's layout).
+// as many lines, lost 0.5 us.) PMAX bounds P: 1 for the loss kernel, 2 for
+// tcgen05, where the warps of a half of the block (a slot, then) issue their
+// products together and must go through the rounds together.
 __host__ __device__ constexpr int cmin(int a, int b) { return a < b ? a : b; }
 
-template <int LX, int LY, bool kPaired = true>
+template <int LX, int LY, int PMAX = kMaxSlots>
 struct FieldLayout {
   static constexpr int NX = 1 << LX;
   static constexpr int NY = 1 << LY;
   static constexpr int TY = NY >> 5;          // threads per column transform
   static constexpr int NGY = kThreads / TY;   // column groups per block
   static constexpr int W = cmin(cmin(8, TY), cmin(NGY, NX));
-  static constexpr int P = (kPaired && W == 8 && 2 * W * TY == kThreads) ? 2 : 1;  // blocks in flight per round
+  // blocks in flight per round
+  static constexpr int P = (W == 8 && W * TY * PMAX >= kThreads) ? kThreads / (W * TY) : 1;
+  // A round of a column pass may keep the next round's blocks in flight in a
+  // second staging buffer: every lane owns a column.
+  static constexpr bool kAhead = W * TY * P == kThreads;
   static constexpr int LW = ilog2(W);
   static constexpr int S = (W == 1) ? 0 : ilog2(16 / W);
   static constexpr int NBLK = NX / W;
   static constexpr int BLOCK = NY * W;        // elements of one column block
   static_assert(P * BLOCK <= 8192, "the column blocks in flight fit the staging buffer");
-  static_assert(P == 1 || W * TY == kThreads / 2, "a slot is half of the block");
+  static_assert(P == 1 || W * TY * P == kThreads, "the slots share out the block");
   __device__ static constexpr int swz(int y) { return W > 1 ? ((y >> S) & (W - 1)) : 0; }
   // element (row y, column x) of the field
   __device__ static size_t off(int y, int x) {
@@ -99,43 +123,124 @@ struct FieldLayout {
   __device__ static int boff(int y, int k) { return y * W + (k ^ swz(y)); }
 };
 
+// The projections of a line's values z, elementwise, after the transform of a
+// pass, and their gaps (part += (|z|/sqrt(N) - a)^2):
+//   kProjTarget  z = Y:       z <- swap(m Y/|Y|)   (Eq. e:Mhat; a = m)
+//   kProjUnit    z = swap(v): z <- v/|v|           (Eq. e:PS with p = 1; a = 1)
+//   kProjSlm     z = swap(v): z <- p v/|v|         (Eq. e:PS; a = p)
+// with the phase of an exact zero taken as 0. amp[stride i] is the amplitude
+// at element i.
+//
+// While every |z|^2 of the thread is a normal number the reciprocal square
+// root is the bare instruction and no zero rule applies: 9-10 instructions per
+// element. Otherwise the loop below it scales subnormals and selects zeros
+// (16 per element); both give the same bits on normal values.
+enum Projection { kProjTarget = 0, kProjUnit = 1, kProjSlm = 2 };
+
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
+template <int PROJ, int V>
+__device__ __forceinline__ void project(float2 (&v)[V], float inv_sqrt_n, const float* amp, int stride, float& part) {
+  auto sq = [](float2 z) {
+    return PROJ == kProjUnit ? norm2(z.y, z.x) : norm2(z.x, z.y);
+  };
+  bool normal = true;
+#pragma unroll
+  for (int i = 0; i < V; ++i) normal &= (sq(v[i]) >= FLT_MIN);  // false for NaN
+  if (normal) {
+#pragma unroll
+    for (int i = 0; i < V; ++i) {
+      const float a = PROJ == kProjUnit ? 1.f : amp[stride * i];
+      const float a2 = sq(v[i]);
+      const float rs = rsqrt_normal(a2);
+      const float d = fmaf(a2 * rs, inv_sqrt_n, -a);
+      part = fmaf(d, d, part);
+      const float f = PROJ == kProjUnit ? rs : a * rs;
+      v[i] = make_float2(v[i].y * f, v[i].x * f);
+    }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < V; ++i) {
+    const float a = PROJ == kProjUnit ? 1.f : amp[stride * i];
+    const float a2 = sq(v[i]);
+    const float rs = rsqrtf(a2);
+    const float mag = a2 > 0.f ? a2 * rs : 0.f;
+    const float d = fmaf(mag, inv_sqrt_n, -a);
+    part = fmaf(d, d, part);
+    const float f = PROJ == kProjUnit ? rs : a * rs;
+    const float2 zero = PROJ == kProjTarget ? make_float2(0.f, a) : make_float2(a, 0.f);
+    v[i] = a2 > 0.f ? make_float2(v[i].y * f, v[i].x * f) : zero;
+  }
+}
+
+// The phases of a thread's values su[STEP i] in (-pi, pi]; a rolled loop
+// holds the only copy of atan2f.
+template <int V, int STEP>
+__device__ __forceinline__ void phase_out(float* po, const float2* su) {
+#pragma unroll 1
+  for (int i = 0; i < V; ++i) {
+    const float2 u = su[STEP * i];
+    const float ph = atan2f(u.y, u.x);
+    po[STEP * i] = (ph <= -3.14159274f) ? 3.14159274f : ph;
+  }
+}
+
 // One pass over rows [lo, hi) (kInit, kRow; LOGN = log2 nx) or column blocks
 // [lo, hi) (kCol, kResid, kInitM; LOGN = log2 ny) of mask mb. Returns this
 // thread's contribution to the pass's gap sum (FP32: the lines it holds).
+//
+// Square grids run rows and columns through this one function body, so that
+// the kernel holds a single copy of the unrolled transform (see project).
 template <int LOGN, int LX, int LY, bool HOLD, class TCF>
 __device__ __forceinline__ float run_pass(const Params& p, int mb, int kind, bool last, int lo, int hi,
                                            unsigned char* smem, Shared& sh, unsigned& mphase,
-                                           const StageTw<LOGN>& tw_rows, const TCF& tcf) {
+                                           const StageTw<LOGN, lane_threads<TCF>()>& tw_rows, const TCF& tcf) {
   // this mask's arrays
   const size_t moff = static_cast<size_t>(mb) * static_cast<size_t>(p.mstride);
   float2* const Bm = p.B + moff;
   const float* const mTm = p.mT + moff;
-  using G = GroupT<LOGN>;
-  using L = FieldLayout<LX, LY>;
+  constexpr int S = lane_threads<TCF>();  // threads per lane
+  constexpr int THR = kThreads * S;
+  using G = GroupT<LOGN, S>;
+  using L = FieldLayout<LX, LY, TCF::kTcgen05 ? 2 : kMaxSlots>;
   constexpr int N = G::N;
   constexpr int T = G::T;
+  constexpr int V = G::V;        // elements per thread: t0 + STEP i
+  constexpr int STEP = G::STEP;
   constexpr int LOGT = LOGN - 5;
   constexpr int LOGNG = 8 - LOGT;  // log2(kThreads / T)
   constexpr int NG = 1 << LOGNG;   // groups per block
-  static_assert(kThreads == 256, "geometry assumes 256 threads");
-  const bool rows = (kind == kInit || kind == kRow);
-  const int g = threadIdx.x >> LOGT;
+  constexpr bool kRows = LOGN == LX, kCols = LOGN == LY;  // the passes this instantiation serves
+  static_assert(kRows || kCols, "lines are rows or columns");
+  static_assert(kThreads == 256, "geometry assumes 256 lanes");
+  const bool rows = kRows && (!kCols || kind == kInit || kind == kRow);
+  const int o = lane_of<S>();  // this thread's lane of the block
+  const int g = o >> LOGT;
   G grp;
-  grp.t = threadIdx.x & (T - 1);
-  grp.bar_id = 1 + g;
+  grp.t = o & (T - 1);
+  grp.c = lane_part<S>();
+  grp.bar_id = 1 + (S == 1 ? g : o / G::TT);
   grp.sm = reinterpret_cast<float2*>(smem) + g * G::SMEM;
+  grp.sx = S == 1 ? nullptr
+                  : reinterpret_cast<float2*>(smem + kSplitSmemOffset) + (o / G::TT) * G::SPLIT + (o & (G::TT - 1));
   grp.tw = rows ? p.twx : p.twy;
-  const int t = grp.t;
+  const int t0 = grp.first();
   // stage twiddles: the kernel's register copy for square grids, else
   // loaded once for this pass
-  StageTw<LOGN> tw_own;
-  if constexpr (!HOLD && !TCF::kEnabled) tw_own.load(grp.tw, t);
-  const StageTw<LOGN>& stw = [&]() -> const StageTw<LOGN>& {
+  StageTw<LOGN, S> tw_own;
+  if constexpr (!HOLD && !TCF::kEnabled) tw_own.load(grp.tw, grp.t, grp.c);
+  const StageTw<LOGN, S>& stw = [&]() -> const StageTw<LOGN, S>& {
     if constexpr (HOLD) return tw_rows;
     else return tw_own;
   }();
   float* ms = reinterpret_cast<float*>(smem + kAmpSmemOffset);
   float2* blk = reinterpret_cast<float2*>(smem + kBlockSmemOffset);
+  const bool from_m = kind == kInitM;  // transform m itself (the target start)
   const int nfft = (kind == kCol || (kind == kRow && !(last && !p.final_resid))) ? 2 : 1;
   const float inv_sqrt_n = p.inv_sqrt_n;
   float acc = 0.f;
@@ -145,7 +250,7 @@ __device__ __forceinline__ float run_pass(const Params& p, int mb, int kind, boo
   // One forward transform of the group's vector: on the FP32 ALUs, on the
   // tensor cores through the warp's slice of the exchange buffers (mma.sync),
   // or on the tensor cores of the block's half (tcgen05, all warps at once).
-  auto fft = [&](float2(&x)[32]) {
+  auto fft = [&](float2(&x)[V]) {
     if constexpr (TCF::kTcgen05) {
       tcf.run(x, tc_in, tc_out);
     } else if constexpr (TCF::kEnabled) {
@@ -154,258 +259,248 @@ __device__ __forceinline__ float run_pass(const Params& p, int mb, int kind, boo
       group_fft<LOGN>(x, grp, stw);
     }
   };
+  // the first line of the threads that transform together: of this warp's
+  // team, or (tcgen05) of this half of the block
+  const int g_first = (TCF::kTcgen05 ? ((o >> 7) << 7) : (o & ~31)) >> LOGT;
 
-  if constexpr (LOGN == LX) {
-  if (rows) {
-    for (int base = lo; base < hi; base += NG) {
-      const int idx = base + g;
-      const bool valid = idx < hi;
-      const int ridx = valid ? idx : base;  // groups past the end work on a valid copy and store nothing
-      float2 v[32];
+  // Column passes: P column blocks (W columns, N = ny rows each) per round,
+  // one per slot of THR / P threads.
+  constexpr int W = L::W;
+  constexpr int P = L::P;
+  constexpr int ST = THR / P;           // threads of a slot
+  constexpr int GS = kThreads / P / T;  // groups of a slot
+  const int slot = P > 1 ? o / (kThreads / P) : 0;
+  const int gl = g - slot * GS;                           // group within the slot
+  const bool gact = gl < W;                               // this group owns a column
+  const int gq = gact ? gl : 0;                           // idle groups read a valid column
+  const bool leader = (threadIdx.x & (ST - 1)) == 0;      // issues the slot's copies
+  const int bi = P - 1 + slot;                            // index of the slot's mbarrier
+  uint64_t* const mbar = &sh.mbar_s[bi];
+  const unsigned pbit = 2u << bi;                         // this mbarrier's phase bit in mphase
+  float* const msl = ms + slot * L::BLOCK;                // the slot's amplitude block
+  float2* bsl = blk + slot * L::BLOCK;                    // the slot's field block
+  // the slot's threads only (the whole block when P == 1)
+  auto slot_sync = [&]() {
+    if constexpr (P > 1) asm volatile("bar.sync %0, %1;" ::"r"(12 + slot), "n"(ST) : "memory");
+    else __syncthreads();
+  };
+  // Rounds after the first find their column block loaded: while a round
+  // transforms one staging buffer, the next round's block lands in the other
+  // (which the store of the round before last has left), and each warp's
+  // amplitude columns are replaced as soon as the warp has projected.
+  const bool ahead = L::kAhead && loads_ahead<TCF>() && !rows && !from_m;
+  // Start the copy of column block cb to the slot's field block `to`, and of
+  // `bytes_m` amplitude bytes that complete on the same phase (leader only).
+  auto load_block = [&](int cb, float2* to, unsigned par, unsigned bytes_m) {
+    bulk_wait_read_all();  // a previous bulk store has read the destination
+    fence_proxy_async_smem();
+    mbar_arrive_expect_tx(mbar, (from_m ? 0u : L::BLOCK * 8u) + bytes_m);
+    if (!from_m) bulk_g2s(to, Bm + static_cast<size_t>(cb) * L::BLOCK, L::BLOCK * 8u, mbar);
+    sh.m_slot[slot] = mTm + static_cast<size_t>(cb) * L::BLOCK;
+    sh.pend_s[bi] = 1;
+    sh.pend_phase_s[bi] = par;
+  };
+  if (!rows && sh.m_layout != P) {  // no amplitude block of another layout stays resident
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int s = 0; s < kMaxSlots; ++s) sh.m_slot[s] = nullptr;
+      sh.m_layout = P;
+    }
+    __syncthreads();
+  }
+  // Row passes of several rounds fetch the next round's rows (16-byte pieces)
+  // into the field staging buffer behind the transforms of this round; a
+  // group's row sits at its own N elements of the buffer.
+  const bool fetch = !TCF::kEnabled && L::W >= 2 && kind == kRow && p.p_slm == nullptr;
+  float2* const next_row = blk + g * N;
+  // the laser amplitude of a row, at this thread's elements (in the field
+  // staging buffer, free in row passes)
+  float* const sp = reinterpret_cast<float*>(blk) + threadIdx.x;
+
+  for (int u0 = lo; u0 < hi; u0 += rows ? NG : P) {
+    const int idx = rows ? u0 + g : u0 + slot;  // this group's row, or this slot's column block
+    float2 v[V];
+    bool work;   // this warp transforms a line in this round
+    bool valid;  // ... and this group's is its own (the others work on a valid copy and store nothing)
+    if (rows) {
+      // Warps without a row leave: transforming copies instead kept the whole
+      // block's issue slots and shared memory busy (256 x 256: row pass 4.3 us
+      // with 2 of 8 warps on rows of their own).
+      if (u0 + g_first >= hi) break;
+      work = true;
+      valid = idx < hi;
+      const int ridx = valid ? idx : u0;
       if (kind == kInit) {
         // exp(i phi) once per run: a rolled loop through the group's exchange
         // buffer keeps a single copy of sincosf (and atan2f) in the kernel.
-        // phi (and p) arrive there first by cp.async, all 32 loads in flight.
-        const float* ph = p.phi_in + moff + static_cast<size_t>(ridx) * N + t;
-        float2* su = grp.sm + t;
-        const float* pp = p.p_slm ? p.p_slm + static_cast<size_t>(ridx) * N + t : nullptr;
+        // phi (and p) arrive there first by cp.async, all loads in flight.
+        const float* ph = p.phi_in + moff + static_cast<size_t>(ridx) * N + t0;
+        float2* su = grp.sm + t0;
+        if constexpr (S > 1) grp.sync();  // the previous round's transform has read the buffer
+        const float* pp = p.p_slm ? p.p_slm + static_cast<size_t>(ridx) * N + t0 : nullptr;
         // rolled: the copies do not wait, so all of them are in flight anyway
 #pragma unroll 1
-        for (int i = 0; i < 32; ++i) cp_async4(&su[T * i].x, ph + T * i);
+        for (int i = 0; i < V; ++i) cp_async4(&su[STEP * i].x, ph + STEP * i);
         if (pp) {
 #pragma unroll 1
-          for (int i = 0; i < 32; ++i) cp_async4(&su[T * i].y, pp + T * i);
+          for (int i = 0; i < V; ++i) cp_async4(&su[STEP * i].y, pp + STEP * i);
         }
         cp_async_wait_all();
 #pragma unroll 1
-        for (int i = 0; i < 32; ++i) {
+        for (int i = 0; i < V; ++i) {
           float s, c;
-          const float2 fa = su[T * i];
+          const float2 fa = su[STEP * i];
           sincosf(fa.x, &s, &c);
           const float a = pp ? fa.y : 1.f;  // u0 = p exp(i phi0)
-          su[T * i] = make_float2(a * c, a * s);
+          su[STEP * i] = make_float2(a * c, a * s);
         }
-        if (last && valid) {  // zero iterations: the mask is arg exp(i phi^0)
-          float* po = p.phi_out + moff + static_cast<size_t>(idx) * N + t;
-#pragma unroll 1
-          for (int i = 0; i < 32; ++i) {
-            const float2 u = su[T * i];
-            const float ph_out = atan2f(u.y, u.x);
-            po[T * i] = (ph_out <= -3.14159274f) ? 3.14159274f : ph_out;
-          }
-        }
+        if (last && valid) phase_out<V, STEP>(p.phi_out + moff + static_cast<size_t>(idx) * N + t0, su);
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = su[T * i];
+        for (int i = 0; i < V; ++i) v[i] = su[STEP * i];
         grp.sync();
       } else {
+        if (fetch && u0 != lo) {
+          cp_async_wait_all();
+          grp.sync();
+          const int flip = L::swz(ridx) & 1;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = Bm[L::off(ridx, t + T * i)];
+          for (int i = 0; i < V; ++i) v[i] = next_row[STEP > 1 ? (t0 ^ flip) + STEP * i : (t0 + i) ^ flip];
+          grp.sync();
+        } else {
+#pragma unroll
+          for (int i = 0; i < V; ++i) v[i] = Bm[L::off(ridx, t0 + STEP * i)];
+        }
+        if (fetch && u0 + NG + g_first < hi) {
+          const int nidx = idx + NG;
+          const int nrow = nidx < hi ? nidx : u0 + NG;
+          // elements x, x + 1 (x even) are 16 bytes of a row segment, in this
+          // order when the row's swizzle is even
+          const int sw = L::swz(nrow) & ~1;
+#pragma unroll 4
+          for (int i = 0; i < V / 2; ++i) {
+            const int x = 2 * (T * S * i + T * grp.c + grp.t);
+            cp_async16(next_row + x, Bm + static_cast<size_t>(x >> L::LW) * L::BLOCK + nrow * L::W +
+                                         ((x & (L::W - 1)) ^ sw));
+          }
+        }
         if (kind == kRow && p.p_slm != nullptr) {
-          // the laser amplitude of this row, prefetched into the (free in
-          // row passes) field staging buffer behind the first transform
-          float* sp = reinterpret_cast<float*>(smem + kBlockSmemOffset) + threadIdx.x;
-          const float* pp = p.p_slm + static_cast<size_t>(ridx) * N + t;
+          // the laser amplitude of this row, prefetched behind the first transform
+          const float* pp = p.p_slm + static_cast<size_t>(ridx) * N + t0;
 #pragma unroll 1
-          for (int i = 0; i < 32; ++i) cp_async4(sp + kThreads * i, pp + T * i);
+          for (int i = 0; i < V; ++i) cp_async4(sp + THR * i, pp + STEP * i);
         }
       }
+    } else {
+      if (idx >= hi) break;  // no block left for this slot
+      work = g_first - slot * GS < W;
+      valid = gact;
+      const unsigned par = (mphase & pbit) ? 1u : 0u;
+      if (ahead) bsl = blk + slot * L::BLOCK + (((u0 - lo) / P) & 1) * kBlockElems;
+      if (!ahead || u0 == lo) {
+        slot_sync();  // the previous round is done with this slot's staging buffers
+        if (leader) {
+          // columns idx W .. idx W + W - 1 of m are contiguous in the transposed
+          // amplitude; a block that stays resident is identified by its global
+          // address, unique across masks and size classes
+          const float* const msrc = mTm + static_cast<size_t>(idx) * L::BLOCK;
+          const unsigned bytes_m = sh.m_slot[slot] != msrc ? L::BLOCK * 4u : 0u;
+          load_block(idx, bsl, par, bytes_m);
+          if (bytes_m) bulk_g2s(msl, msrc, bytes_m, mbar);
+        }
+      }
+      const bool landed = mbar_wait_bounded(mbar, par);
+      mphase ^= pbit;
+      if (!landed) {
+        fail(p, GS_ETIMEOUT);
+      } else if (leader) {
+        sh.pend_s[bi] = 0;
+      }
+      if (from_m) {
+        // The target start transforms m itself: stage swap((m, 0)) in the field
+        // layout, so the forward DFT below yields swap(IDFT_y(m)).
+        for (int e = threadIdx.x & (ST - 1); e < L::BLOCK; e += ST) {
+          const int k = e % W;
+          const int y = e / W;
+          bsl[L::boff(y, k)] = make_float2(0.f, msl[k * L::NY + y]);
+        }
+        slot_sync();
+      }
+      if (work) {
+#pragma unroll
+        for (int i = 0; i < V; ++i) v[i] = bsl[L::boff(t0 + STEP * i, gq)];
+      }
+    }
 
+    if (work) {
       float part = 0.f;
 #pragma unroll 1
       for (int h = 0; h < nfft; ++h) {
         fft(v);
-        if (h != 0 || kind != kRow) continue;
-        // v = swap(IDFT_x(B)) = swap(sqrt(N) P_M u^nu). Gap to S and Eq. (e:PS).
-        if (p.p_slm == nullptr) {  // p = 1
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const float vx = v[i].y;
-            const float vy = v[i].x;
-            const float a2 = vx * vx + vy * vy;
-            const float rs = rsqrtf(a2);
-            const float mag = a2 > 0.f ? a2 * rs : 0.f;
-            const float d = mag * inv_sqrt_n - 1.f;
-            part += d * d;
-            v[i] = a2 > 0.f ? make_float2(vx * rs, vy * rs) : make_float2(1.f, 0.f);
+        if (h != 0) continue;
+        if (rows) {
+          if (kind != kRow) continue;
+          // v = swap(IDFT_x(B)) = swap(sqrt(N) P_M u^nu). Gap to S and Eq. (e:PS).
+          if (p.p_slm == nullptr) {
+            project<kProjUnit, V>(v, inv_sqrt_n, nullptr, 0, part);
+          } else {
+            cp_async_wait_all();
+            project<kProjSlm, V>(v, inv_sqrt_n, sp, THR, part);
           }
-        } else {
-          // SLM amplitude p: u = p v/|v|, gap |P_M u| - p. A rolled loop
-          // through the group's exchange buffer keeps this variant out of the
-          // unrolled hot code.
-          float2* su = grp.sm + t;
-          const float* sp = reinterpret_cast<const float*>(smem + kBlockSmemOffset) + threadIdx.x;
+          if (last) {
+            // The mask, once per run: through the group's exchange buffer so
+            // that a rolled loop holds the only copy of atan2f.
+            float2* su = grp.sm + t0;
+            if constexpr (S > 1) grp.sync();  // the transform has read the buffer
 #pragma unroll
-          for (int i = 0; i < 32; ++i) su[T * i] = v[i];
-          cp_async_wait_all();
-#pragma unroll 1
-          for (int i = 0; i < 32; ++i) {
-            const float a = sp[kThreads * i];
-            const float2 w = su[T * i];
-            const float vx = w.y;
-            const float vy = w.x;
-            const float a2 = vx * vx + vy * vy;
-            const float rs = rsqrtf(a2);
-            const float mag = a2 > 0.f ? a2 * rs : 0.f;
-            const float d = mag * inv_sqrt_n - a;
-            part += d * d;
-            const float f = a * rs;
-            su[T * i] = a2 > 0.f ? make_float2(vx * f, vy * f) : make_float2(a, 0.f);
+            for (int i = 0; i < V; ++i) su[STEP * i] = v[i];
+            if (valid) phase_out<V, STEP>(p.phi_out + moff + static_cast<size_t>(idx) * N + t0, su);
+            grp.sync();
           }
-#pragma unroll
-          for (int i = 0; i < 32; ++i) v[i] = su[T * i];
-          grp.sync();  // the buffer is reused by the next transform's exchange
-        }
-        if (last) {
-          // The mask, once per run: through the group's exchange buffer so
-          // that a rolled loop holds the only copy of atan2f.
-          float2* su = grp.sm + t;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) su[T * i] = v[i];
-          if (valid) {
-            float* po = p.phi_out + moff + static_cast<size_t>(idx) * N + t;
-#pragma unroll 1
-            for (int i = 0; i < 32; ++i) {
-              const float2 u = su[T * i];
-              const float ph_out = atan2f(u.y, u.x);
-              po[T * i] = (ph_out <= -3.14159274f) ? 3.14159274f : ph_out;
+        } else if (!from_m) {
+          // v = Y = F u^nu along this column. Residual and Eq. (e:Mhat); the
+          // result is swapped, so the next forward DFT acts as the inverse
+          // (kResid ends here and ignores it).
+          project<kProjTarget, V>(v, inv_sqrt_n, msl + gq * N + t0, STEP, part);
+          if (ahead && idx + P < hi) {
+            // the next round's block; its amplitude columns replace those of
+            // the lines that transform together, which have read theirs
+            if (leader) {
+              float2* const other = blk + slot * L::BLOCK + ((((u0 - lo) / P) & 1) ^ 1) * kBlockElems;
+              load_block(idx + P, other, (mphase & pbit) ? 1u : 0u, L::BLOCK * 4u);
+            }
+            grp.sync();
+            if ((o & (G::TT - 1)) == 0) {
+              fence_proxy_async_smem();
+              const int k = g_first - slot * GS;  // the team's first column
+              bulk_g2s(msl + k * N, mTm + (static_cast<size_t>(idx + P) * W + k) * N, G::TT * 32 * 4u, mbar);
             }
           }
-          grp.sync();
         }
       }
-      if (valid) acc += part;
-      if (valid && (kind == kInit || nfft == 2)) {
+      if (valid) {
+        acc += part;
+        if (rows) {
+          if (kind == kInit || nfft == 2) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) Bm[L::off(idx, t + T * i)] = v[i];
-      }
-    }
-    return acc;
-  }
-  }
-
-  // Column passes: P column blocks (W columns, N = ny rows each) per round,
-  // one per slot of kThreads / P threads.
-  if constexpr (LOGN == LY) {
-  constexpr int W = L::W;
-  constexpr int P = L::P;
-  constexpr int ST = kThreads / P;  // threads of a slot
-  constexpr int GS = ST / T;        // groups of a slot
-  static_assert(N == L::NY, "column transforms have length ny");
-  const int slot = (P == 2) ? static_cast<int>(threadIdx.x >> 7) : 0;
-  const int gl = g - slot * GS;                           // group within the slot
-  const bool gact = gl < W;                               // this group owns a column
-  // some group of this warp owns a column (tcgen05: of this half of the
-  // block, whose warps issue their products together)
-  const int w_first = (TCF::kTcgen05 ? (((threadIdx.x >> 7) << 7) >> LOGT) : ((threadIdx.x & ~31) >> LOGT)) - slot * GS;
-  const bool wact = w_first < W;
-  const int gq = gact ? gl : 0;                           // idle groups read a valid column
-  const bool leader = (threadIdx.x & (ST - 1)) == 0;      // issues the slot's copies
-  uint64_t* const mbar = (P == 2) ? &sh.mbar_s[slot] : &sh.mbar;
-  const unsigned pbit = (P == 2) ? (2u << slot) : 1u;     // this mbarrier's phase bit in mphase
-  float* const msl = ms + slot * L::BLOCK;                // the slot's amplitude block
-  float2* const bsl = blk + slot * L::BLOCK;              // the slot's field block
-  // the slot's threads only (the whole block when P == 1)
-  auto slot_sync = [&]() {
-    if constexpr (P == 2) asm volatile("bar.sync %0, %1;" ::"r"(14 + slot), "n"(ST) : "memory");
-    else __syncthreads();
-  };
-  for (int cb0 = lo; cb0 < hi; cb0 += P) {
-    const int cb = cb0 + slot;
-    if (cb >= hi) break;  // P = 2: no block left for this slot
-    slot_sync();  // the previous round is done with this slot's staging buffers
-    const bool from_m = (kind == kInitM);  // transform m itself (the target start)
-    const unsigned par = (mphase & pbit) ? 1u : 0u;
-    if (leader) {
-      bulk_wait_read_all();  // a previous bulk store has read the slot's field block
-      fence_proxy_async_smem();
-      // the amplitude block is identified by its global address, unique
-      // across masks and size classes; the regions of the two layouts of the
-      // staging buffer overlap, so loading one invalidates the others
-      const float* const msrc = mTm + static_cast<size_t>(cb) * L::BLOCK;
-      const float*& resident = (P == 2) ? sh.m_slot[slot] : sh.m_block;
-      const bool need_m = (resident != msrc);
-      const unsigned bytes_b = from_m ? 0u : L::BLOCK * 8u;
-      const unsigned bytes_m = L::BLOCK * 4u;
-      mbar_arrive_expect_tx(mbar, bytes_b + (need_m ? bytes_m : 0u));
-      if (!from_m) bulk_g2s(bsl, Bm + static_cast<size_t>(cb) * L::BLOCK, bytes_b, mbar);
-      // columns cb W .. cb W + W - 1 of m are contiguous in the transposed amplitude
-      if (need_m) {
-        bulk_g2s(msl, mTm + static_cast<size_t>(cb) * L::BLOCK, bytes_m, mbar);
-        if constexpr (P == 2) sh.m_block = nullptr;
-        else sh.m_slot[0] = sh.m_slot[1] = nullptr;
-      }
-      resident = msrc;
-      if constexpr (P == 2) {
-        sh.pend_s[slot] = 1;
-        sh.pend_phase_s[slot] = par;
-      } else {
-        sh.pending = 1;
-        sh.pending_phase = par;
-      }
-    }
-    const bool landed = mbar_wait_bounded(mbar, par);
-    mphase ^= pbit;
-    if (!landed) {
-      fail(p, GS_ETIMEOUT);
-    } else if (leader) {
-      if constexpr (P == 2) sh.pend_s[slot] = 0;
-      else sh.pending = 0;
-    }
-    if (from_m) {
-      // The target start transforms m itself: stage swap((m, 0)) in the field
-      // layout, so the forward DFT below yields swap(IDFT_y(m)).
-      for (int e = threadIdx.x & (ST - 1); e < L::BLOCK; e += ST) {
-        const int k = e % W;
-        const int y = e / W;
-        bsl[L::boff(y, k)] = make_float2(0.f, msl[k * N + y]);
-      }
-      slot_sync();
-    }
-    if (wact) {
-      float2 v[32];
-#pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = bsl[L::boff(t + T * i, gq)];
-      float part = 0.f;
-#pragma unroll 1
-      for (int h = 0; h < nfft; ++h) {
-        fft(v);
-        if (h != 0 || from_m) continue;
-        // v = Y = F u^nu along this column. Residual and Eq. (e:Mhat).
-        const float* mcol = msl + gq * N + t;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const float m = mcol[T * i];
-          const float2 Y = v[i];
-          const float a2 = Y.x * Y.x + Y.y * Y.y;
-          const float rs = rsqrtf(a2);
-          const float mag = a2 > 0.f ? a2 * rs : 0.f;
-          const float d = mag * inv_sqrt_n - m;
-          part += d * d;
-          if (kind == kCol) {
-            const float f = m * rs;
-            const float2 Yh = a2 > 0.f ? make_float2(Y.x * f, Y.y * f) : make_float2(m, 0.f);
-            v[i] = make_float2(Yh.y, Yh.x);  // swapped: the next forward DFT acts as the inverse
+            for (int i = 0; i < V; ++i) Bm[L::off(idx, t0 + STEP * i)] = v[i];
           }
+        } else if (kind != kResid) {
+#pragma unroll
+          for (int i = 0; i < V; ++i) bsl[L::boff(t0 + STEP * i, gl)] = v[i];
         }
       }
-      if (gact) acc += part;
-      if ((kind == kCol || from_m) && gact) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) bsl[L::boff(t + T * i, gl)] = v[i];
-      }
     }
-    if (kind == kCol || from_m) {
+    if (!rows && (kind != kResid || ahead)) {
       slot_sync();
-      if (leader) {
+      if (kind != kResid && leader) {
         fence_proxy_async_smem();
-        bulk_s2g(Bm + static_cast<size_t>(cb) * L::BLOCK, bsl, L::BLOCK * 8u);
+        bulk_s2g(Bm + static_cast<size_t>(idx) * L::BLOCK, bsl, L::BLOCK * 8u);
         bulk_commit();
       }
     }
   }
   // the field must be in global memory before the grid barrier releases the next pass
-  if ((kind == kCol || kind == kInitM) && leader) bulk_wait_all();
-  }
+  if (!rows && kind != kResid && leader) bulk_wait_all();
   return acc;
 }
 
@@ -413,8 +508,8 @@ __device__ __forceinline__ float run_pass(const Params& p, int mb, int kind, boo
 // block's shared memory a bounded time to land.
 static __device__ void drain_copies(Shared& sh) {
   if (threadIdx.x == 0 && sh.pending) mbar_wait_bounded(&sh.mbar, sh.pending_phase);
-  for (int s = 0; s < 2; ++s)
-    if (threadIdx.x == 128u * s && sh.pend_s[s]) mbar_wait_bounded(&sh.mbar_s[s], sh.pend_phase_s[s]);
+  if (threadIdx.x < kSlotBars && sh.pend_s[threadIdx.x])
+    mbar_wait_bounded(&sh.mbar_s[threadIdx.x], sh.pend_phase_s[threadIdx.x]);
   __syncthreads();
 }
 
@@ -432,13 +527,13 @@ static __device__ void build_amplitude(const Params& p, int mb, float s, unsigne
   for (int base = lo; base < hi; base += W) {
     const int wcur = min(W, hi - base);
     __syncthreads();
-    for (int e = threadIdx.x; e < p.ny * W; e += kThreads) {
+    for (int e = threadIdx.x; e < p.ny * W; e += blockDim.x) {
       const int k = e & (W - 1);
       const int y = e >> logNG;
       if (k < wcur) blk[y * (W + 1) + k] = Im[static_cast<size_t>(y) * p.nx + base + k];
     }
     __syncthreads();
-    for (int e = threadIdx.x; e < wcur * p.ny; e += kThreads) {
+    for (int e = threadIdx.x; e < wcur * p.ny; e += blockDim.x) {
       const int k = e >> p.logny;
       const int y = e & (p.ny - 1);
       mTm[static_cast<size_t>(base + k) * p.ny + y] = s * sqrtf(blk[y * (W + 1) + k]);
@@ -466,7 +561,7 @@ static __device__ __forceinline__ void a0_partials(const Params& p, Shared& sh) 
     const float* I = p.I + static_cast<size_t>(mb) * static_cast<size_t>(p.mstride) + static_cast<size_t>(r0) * p.nx;
     double acc = 0.0;
     bool bad = false;
-    for (int e = threadIdx.x; e < cnt; e += kThreads) {
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
       const float x = I[e];
       bad |= !(x >= 0.f && x <= FLT_MAX);
       acc += static_cast<double>(x);
@@ -508,9 +603,9 @@ static __device__ __forceinline__ int a0_scales(const Params& p, Shared& sh, int
     for (int mb = 0; mb < p.batch; ++mb) {
       if (!sh.bad[base + mb]) continue;
       if (p.r_out)
-        for (int e = threadIdx.x; e < nr; e += kThreads) p.r_out[static_cast<size_t>(mb) * p.rstride + e] = nan;
+        for (int e = threadIdx.x; e < nr; e += blockDim.x) p.r_out[static_cast<size_t>(mb) * p.rstride + e] = nan;
       if (p.g_out)
-        for (int e = threadIdx.x; e < p.iters; e += kThreads) p.g_out[static_cast<size_t>(mb) * p.gstride + e] = nan;
+        for (int e = threadIdx.x; e < p.iters; e += blockDim.x) p.g_out[static_cast<size_t>(mb) * p.gstride + e] = nan;
     }
   }
   return nbad;
@@ -526,7 +621,7 @@ template <int LX, int LY = LX>
 __device__ __forceinline__ void build_amplitudes(const Params& p, Shared& sh, int base, unsigned char* smem) {
   for (int mb = 0; mb < p.batch; ++mb)
     if (!sh.bad[base + mb]) {
-      if constexpr (LX == 0) gen_build_amplitude(p, mb, sh.scale[base + mb]);
+      if constexpr (LX == 0) gen_build_amplitude(p, mb, sh.scale[base + mb], smem);
       else if constexpr (is_rg_side(LX)) rg_build_amplitude<LX, LY>(p, mb, sh.scale[base + mb], smem);
       else build_amplitude(p, mb, sh.scale[base + mb], smem);
     }
@@ -571,14 +666,20 @@ static __device__ __forceinline__ PassInfo pass_info(const Params& p, int q0) {
 // masks (rows, or column blocks) form one sequence split evenly over the
 // blocks, so that small masks of a batch do not leave blocks idle; a block
 // works through its share mask by mask and writes the FP64 partial of each
-// mask's gap to its slot (zero for the masks it does not touch).
+// mask's gap to its slot (zero for the masks it does not touch). With `late`
+// the last mask's sum is left to the barrier that follows (grid_sync).
+struct LateSum {
+  float x = 0.f;
+  double* to = nullptr;
+};
 template <int LX, int LY, bool HOLD, class TCF, class TW>
-__device__ __forceinline__ void class_pass(const Params& p, Shared& sh, int base, int w0, int w1, const PassInfo& f,
-                                           unsigned char* smem, unsigned& mphase, const TW& tw_rows,
-                                           const TCF& tcf) {
+__device__ __forceinline__ LateSum class_pass(const Params& p, Shared& sh, int base, int w0, int w1,
+                                              const PassInfo& f, bool late, unsigned char* smem, unsigned& mphase,
+                                              const TW& tw_rows, const TCF& tcf) {
+  LateSum left;
   const bool rows = (f.kind == kInit || f.kind == kRow);
   int per;  // units of one mask
-  if constexpr (LX == 0) per = rows ? p.ny : (p.nx + kGenTeams - 1) / kGenTeams;
+  if constexpr (LX == 0) per = rows ? p.ny : p.nx;
   else if constexpr (is_rg_side(LX)) per = rows ? p.ny : LX / RgLayout<LX, LY>::W;
   else per = rows ? p.ny : FieldLayout<LX, LY>::NBLK;
   const int G = gridDim.x;
@@ -610,15 +711,22 @@ __device__ __forceinline__ void class_pass(const Params& p, Shared& sh, int base
     } else if constexpr (LX == LY) {
       a = run_pass<LX, LX, LY, HOLD>(p, mb, f.kind, f.last, slo, shi, smem, sh, mphase, tw_rows, tcf);
     } else {
-      const StageTw<LY> none{};
+      const StageTw<LY, lane_threads<TCF>()> none{};
       a = rows ? run_pass<LX, LX, LY, false>(p, mb, f.kind, f.last, slo, shi, smem, sh, mphase, tw_rows, tcf)
                : run_pass<LY, LX, LY, false>(p, mb, f.kind, f.last, slo, shi, smem, sh, mphase, none, tcf);
     }
     if (f.slot >= 0) {
-      const double tot = block_sum_f(a, sh);
-      if (threadIdx.x == 0) p.partials[(static_cast<size_t>(f.slot) * p.batch + mb) * G + blockIdx.x] = tot;
+      double* const to = p.partials + (static_cast<size_t>(f.slot) * p.batch + mb) * G + blockIdx.x;
+      if (late && mb == m1 - 1) {
+        left.x = a;
+        left.to = to;
+      } else {
+        const double tot = block_sum_f(a, sh);
+        if (threadIdx.x == 0) *to = tot;
+      }
     }
   }
+  return left;
 }
 
 // Gaps: r from column passes, g from row passes, in FP64, for every valid
@@ -655,13 +763,15 @@ static __device__ __forceinline__ void final_gaps(const Params& p, Shared& sh, i
 static __device__ __forceinline__ void block_setup(Shared& sh) {
   if (threadIdx.x == 0) {
     mbar_init(&sh.mbar, 1);
-    mbar_init(&sh.mbar_s[0], 1);
-    mbar_init(&sh.mbar_s[1], 1);
+    for (int s = 0; s < kSlotBars; ++s) {
+      mbar_init(&sh.mbar_s[s], 1);
+      sh.pend_s[s] = 0;
+    }
     fence_barrier_init();
     sh.pending = 0;
     sh.m_block = nullptr;
-    sh.m_slot[0] = sh.m_slot[1] = nullptr;
-    sh.pend_s[0] = sh.pend_s[1] = 0;
+    for (int s = 0; s < kMaxSlots; ++s) sh.m_slot[s] = nullptr;
+    sh.m_layout = 0;
   }
   __syncthreads();
 }
@@ -702,11 +812,13 @@ __device__ __forceinline__ void iterate_class(const Params& p, Shared& sh, unsig
   for (int w0 = 0; w0 < p.batch; w0 += gsz) {  // mask groups, each through the whole schedule
     const int w1 = min(p.batch, w0 + gsz);
     for (int q0 = 0; q0 < npass; ++q0) {
-      class_pass<LX, LY, kHold>(p, sh, 0, w0, w1, pass_info(p, q0), smem, mphase, tw_rows, tcf);
+      // the sums of the last pass are read right after its barrier
+      const LateSum ls =
+          class_pass<LX, LY, kHold>(p, sh, 0, w0, w1, pass_info(p, q0), q0 + 1 < npass, smem, mphase, tw_rows, tcf);
       // pass timestamps: work done, then released by the barrier
       unsigned long long* const trq = tr ? tr + static_cast<size_t>(2 * (1 + q0)) * gridDim.x : nullptr;
       if (trq) trq[0] = global_ns();
-      if (!grid_sync(p, target, sh)) {
+      if (!grid_sync(p, target, sh, ls.x, ls.to)) {
         drain_copies(sh);
         return;
       }
@@ -716,15 +828,23 @@ __device__ __forceinline__ void iterate_class(const Params& p, Shared& sh, unsig
   final_gaps(p, sh, 0);
 }
 
+template <int LX, int LY, bool TC>
+__host__ __device__ constexpr int kernel_split() {
+  return (TC || LX == 0) ? 1 : iteration_split(1 << LX, 1 << LY);
+}
+
 // One size class per launch (every grid).
 template <int LX, int LY, bool TC = false>
-__global__ void __launch_bounds__(kThreads, 1) gs_iterate(const Params p) {
+__global__ void __launch_bounds__(LX == 0 ? kGenMaxThreads : kThreads * kernel_split<LX, LY, TC>(), 1) gs_iterate(const Params p) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Shared sh;
   if (*reinterpret_cast<volatile int*>(p.abort_flag) != 0) return;  // an earlier chunk failed
   constexpr bool kHold = LX > 0 && LX == LY && !TC;
-  StageTw<LX> tw_rows;  // square grids: stage twiddles held for the whole run
-  if constexpr (kHold) tw_rows.load(p.twx, threadIdx.x & ((1 << (LX - 5)) - 1));
+  constexpr int S = kernel_split<LX, LY, TC>();
+  StageTw<LX, S> tw_rows;  // square grids: stage twiddles held for the whole run
+  if constexpr (kHold) {
+    tw_rows.load(p.twx, lane_of<S>() & ((1 << (LX - 5)) - 1), lane_part<S>());
+  }
   // Tensor-core transforms: the block's tables, then the DFT-matrix fragments
   // held in registers for the whole run.
   static_assert(!TC || LX == LY, "tensor-core kernels are square");
@@ -740,7 +860,7 @@ __global__ void __launch_bounds__(kThreads, 1) gs_iterate(const Params p) {
   }
   const auto tcf = [&]() {
     if constexpr (TC) return TcFft<LX>{s1, s2, tctw};
-    else return NoTc{};
+    else return NoTc<S>{};
   }();
   iterate_class<LX, LY, kHold>(p, sh, smem, tw_rows, tcf);
 }
@@ -783,18 +903,18 @@ __global__ void __launch_bounds__(kThreads, 1) gs_iterate_tc5(const Params p) {
 }
 
 template <int C, bool TC>
-__device__ __forceinline__ void mixed_class_pass(const MixedParams& mp, Shared& sh, int w0, int w1, const PassInfo& f,
-                                                 unsigned char* smem, unsigned& mphase, const TcStage1& s1,
+__device__ __forceinline__ LateSum mixed_class_pass(const MixedParams& mp, Shared& sh, int w0, int w1,
+                                                    const PassInfo& f, bool late, unsigned char* smem, unsigned& mphase, const TcStage1& s1,
                                                  const TcStage2<8 << C>& s2) {
   constexpr int L = 8 + C;
   const Params& p = mp.cls[C];
   const int base = (C > 0 ? mp.cls[0].batch : 0) + (C > 1 ? mp.cls[1].batch : 0);
-  const StageTw<L> none{};
+  const StageTw<L, TC ? 1 : kMixedSplit> none{};
   if constexpr (TC) {
     const TcFft<L> tcf{s1, s2, reinterpret_cast<const float2*>(smem + kTcTwOffset + C * kTcTwBytes)};
-    class_pass<L, L, false>(p, sh, base, w0, w1, f, smem, mphase, none, tcf);
+    return class_pass<L, L, false>(p, sh, base, w0, w1, f, late, smem, mphase, none, tcf);
   } else {
-    class_pass<L, L, false>(p, sh, base, w0, w1, f, smem, mphase, none, NoTc{});
+    return class_pass<L, L, false>(p, sh, base, w0, w1, f, late, smem, mphase, none, NoTc<kMixedSplit>{});
   }
 }
 
@@ -842,8 +962,8 @@ __device__ __forceinline__ void iterate_mixed(const MixedParams& mp, Shared& sh,
     for (int w0 = 0; w0 < pc.batch; w0 += gsz) {
       const int w1 = min(pc.batch, w0 + gsz);
       for (int q0 = 0; q0 < npass; ++q0) {
-        pass(c, w0, w1, pass_info(p0, q0), mphase);
-        if (!grid_sync(p0, target, sh)) {
+        const LateSum ls = pass(c, w0, w1, pass_info(p0, q0), q0 + 1 < npass, mphase);
+        if (!grid_sync(p0, target, sh, ls.x, ls.to)) {
           drain_copies(sh);
           return;
         }
@@ -856,7 +976,7 @@ __device__ __forceinline__ void iterate_mixed(const MixedParams& mp, Shared& sh,
 }
 
 template <bool TC>
-__global__ void __launch_bounds__(kThreads, 1) gs_iterate_mixed(const MixedParams mp) {
+__global__ void __launch_bounds__(TC ? kThreads : kThreads * kMixedSplit, 1) gs_iterate_mixed(const MixedParams mp) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Shared sh;
   if (*reinterpret_cast<volatile int*>(mp.cls[0].abort_flag) != 0) return;
@@ -910,10 +1030,12 @@ __global__ void __launch_bounds__(kThreads, 1) gs_iterate_mixed(const MixedParam
       const int w1 = min(pc.batch, w0 + gsz);
       for (int q0 = 0; q0 < npass; ++q0) {
         const PassInfo f = pass_info(p0, q0);
-        if (c == 0) mixed_class_pass<0, TC>(mp, sh, w0, w1, f, smem, mphase, s1, s2a);
-        else if (c == 1) mixed_class_pass<1, TC>(mp, sh, w0, w1, f, smem, mphase, s1, s2b);
-        else mixed_class_pass<2, TC>(mp, sh, w0, w1, f, smem, mphase, s1, s2c);
-        if (!grid_sync(p0, target, sh)) {
+        const bool late = q0 + 1 < npass;
+        LateSum ls;
+        if (c == 0) ls = mixed_class_pass<0, TC>(mp, sh, w0, w1, f, late, smem, mphase, s1, s2a);
+        else if (c == 1) ls = mixed_class_pass<1, TC>(mp, sh, w0, w1, f, late, smem, mphase, s1, s2b);
+        else ls = mixed_class_pass<2, TC>(mp, sh, w0, w1, f, late, smem, mphase, s1, s2c);
+        if (!grid_sync(p0, target, sh, ls.x, ls.to)) {
           drain_copies(sh);
           return;
         }
@@ -937,13 +1059,13 @@ constexpr int kMixedTwOffset = 4 * tc5_form_bytes(32) + 2 * tc5_form_bytes(8) + 
 static_assert(kMixedTwOffset + 3 * kTc5TwBytes == kMixedTc5ExtraSmemBytes, "mixed tcgen05 tables match the launch size");
 
 template <int C, bool BF16>
-__device__ __forceinline__ void mixed_class_pass_tc5(const MixedParams& mp, Shared& sh, int w0, int w1,
-                                                     const PassInfo& f, unsigned char* smem, unsigned& mphase,
+__device__ __forceinline__ LateSum mixed_class_pass_tc5(const MixedParams& mp, Shared& sh, int w0, int w1,
+                                                     const PassInfo& f, bool late, unsigned char* smem, unsigned& mphase,
                                                      const Tc5Fft<8 + C, BF16>& tcf) {
   constexpr int L = 8 + C;
   const int base = (C > 0 ? mp.cls[0].batch : 0) + (C > 1 ? mp.cls[1].batch : 0);
   const StageTw<L> none{};
-  class_pass<L, L, false>(mp.cls[C], sh, base, w0, w1, f, smem, mphase, none, tcf);
+  return class_pass<L, L, false>(mp.cls[C], sh, base, w0, w1, f, late, smem, mphase, none, tcf);
 }
 
 template <bool BF16>
@@ -975,10 +1097,10 @@ __global__ void __launch_bounds__(kThreads, 1) gs_iterate_mixed_tc5(const MixedP
   const Tc5Fft<8, BF16> t8{smem, b1, smem_u32(tabs + mixed_b2_offset(0)), tw, tc_mbar, tc_tmem, &phase, &p0};
   const Tc5Fft<9, BF16> t9{smem, b1, smem_u32(tabs + mixed_b2_offset(1)), tw + 1024, tc_mbar, tc_tmem, &phase, &p0};
   const Tc5Fft<10, BF16> t10{smem, b1, smem_u32(tabs + mixed_b2_offset(2)), tw + 2048, tc_mbar, tc_tmem, &phase, &p0};
-  iterate_mixed(mp, sh, smem, [&](int c, int w0, int w1, const PassInfo& f, unsigned& mphase) {
-    if (c == 0) mixed_class_pass_tc5<0, BF16>(mp, sh, w0, w1, f, smem, mphase, t8);
-    else if (c == 1) mixed_class_pass_tc5<1, BF16>(mp, sh, w0, w1, f, smem, mphase, t9);
-    else mixed_class_pass_tc5<2, BF16>(mp, sh, w0, w1, f, smem, mphase, t10);
+  iterate_mixed(mp, sh, smem, [&](int c, int w0, int w1, const PassInfo& f, bool late, unsigned& mphase) {
+    if (c == 0) return mixed_class_pass_tc5<0, BF16>(mp, sh, w0, w1, f, late, smem, mphase, t8);
+    if (c == 1) return mixed_class_pass_tc5<1, BF16>(mp, sh, w0, w1, f, late, smem, mphase, t9);
+    return mixed_class_pass_tc5<2, BF16>(mp, sh, w0, w1, f, late, smem, mphase, t10);
   });
   tc5_fence_before();
   __syncthreads();

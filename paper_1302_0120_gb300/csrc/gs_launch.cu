@@ -99,14 +99,23 @@ static const void* kernel_for(int nx, int ny, int tc_mode) {
   }
 }
 
+// threads per block of the kernel of an nx x ny grid (not the general kernel,
+// whose block depends on the run)
+static int iteration_threads(int nx, int ny, int tc_mode) {
+  return (uses_general(nx, ny) || tc_mode != kTcNone) ? kThreads : kThreads * iteration_split(nx, ny);
+}
+
+static int mixed_threads(int tc_mode) { return tc_mode != kTcNone ? kThreads : kThreads * kMixedSplit; }
+
 size_t iteration_smem_bytes(int nx, int ny, int tc_mode) {
   if (uses_rg(nx, ny)) return rg_smem_bytes(nx, ny);
-  if (uses_general(nx, ny)) return gen_smem_bytes(nx, ny);
+  if (uses_general(nx, ny)) return gen_smem_bytes(nx, ny, 4);
   // group exchange buffers, one column block of the amplitude, one of the
-  // field; then the tensor-core tables (and, for tcgen05, operands)
+  // field; then the split-exchange buffers, or the tensor-core tables (and,
+  // for tcgen05, operands)
   const size_t extra = tc_mode == kTcMmaSync ? kTcExtraSmemBytes
                        : (tc_mode == kTcGen05F16 || tc_mode == kTcGen05Bf16) ? kTc5ExtraSmemBytes
-                                                                               : 0;
+                                                                               : lane_smem_bytes(iteration_split(nx, ny));
   return kGroupSmemBytes + 8192 * 4 + 8192 * 8 + extra;
 }
 
@@ -116,10 +125,10 @@ cudaError_t iteration_occupancy(int nx, int ny, int* blocks_per_sm, int tc_mode)
   const size_t smem = iteration_smem_bytes(nx, ny, tc_mode);
   // The general kernel serves every size: allow its largest request, so that
   // contexts of different sizes do not undo each other's setting.
-  const size_t allow = (uses_general(nx, ny) && !uses_rg(nx, ny)) ? gen_smem_bytes(kMaxGeneralSide, kMaxGeneralSide) : smem;
+  const size_t allow = (uses_general(nx, ny) && !uses_rg(nx, ny)) ? kGenSmemLimit : smem;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(allow));
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kThreads, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, iteration_threads(nx, ny, tc_mode), smem);
 }
 
 size_t mixed_smem_bytes(int tc_mode) {
@@ -127,7 +136,7 @@ size_t mixed_smem_bytes(int tc_mode) {
   // tcgen05: the matrices and twiddle tables of the three lengths
   const size_t extra = tc_mode == kTcMmaSync ? 3 * 32 * 32 * 8 + 32 * 8
                        : (tc_mode == kTcGen05F16 || tc_mode == kTcGen05Bf16) ? kMixedTc5ExtraSmemBytes
-                                                                               : 0;
+                                                                               : lane_smem_bytes(kMixedSplit);
   return kGroupSmemBytes + 8192 * 4 + 8192 * 8 + extra;
 }
 
@@ -136,21 +145,24 @@ cudaError_t mixed_occupancy(int tc_mode, int* blocks_per_sm) {
   const size_t smem = mixed_smem_bytes(tc_mode);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, kThreads, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, mixed_threads(tc_mode), smem);
 }
 
 cudaError_t launch_mixed(const MixedParams& mp, int grid, int tc_mode, cudaStream_t s) {
   void* args[] = {const_cast<MixedParams*>(&mp)};
-  return cudaLaunchCooperativeKernel(iterate_kernel_mixed(tc_mode), dim3(grid), dim3(kThreads), args,
+  return cudaLaunchCooperativeKernel(iterate_kernel_mixed(tc_mode), dim3(grid), dim3(mixed_threads(tc_mode)), args,
                                      mixed_smem_bytes(tc_mode), s);
 }
 
 cudaError_t launch_iterations(const Params& p, int grid, cudaStream_t s) {
   const void* k = kernel_for(p.nx, p.ny, p.tensor_core);
   if (k == nullptr) return cudaErrorInvalidValue;
-  const size_t smem = iteration_smem_bytes(p.nx, p.ny, p.tensor_core);
   void* args[] = {const_cast<Params*>(&p)};
-  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads), args, smem, s);
+  if (p.gen_teams > 0)
+    return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(p.gen_teams << p.gen_team_log), args,
+                                       gen_smem_bytes(p.nx, p.ny, p.gen_teams), s);
+  const size_t smem = iteration_smem_bytes(p.nx, p.ny, p.tensor_core);
+  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(iteration_threads(p.nx, p.ny, p.tensor_core)), args, smem, s);
 }
 
 }  // namespace gsk

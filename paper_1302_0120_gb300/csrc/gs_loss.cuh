@@ -81,26 +81,32 @@ static __device__ bool loss_sync(const LossParams& p, unsigned& target, Shared& 
 // kLossPrepare launch); with the Adam update, p.steps optimiser steps.
 
 template <int LN, int MODE>
-__global__ void __launch_bounds__(kThreads, 1) gs_loss_kernel(const LossParams p) {
-  using G = GroupT<LN>;
-  using L = FieldLayout<LN, LN, false>;
+__global__ void __launch_bounds__(kThreads * kLossSplit, 1) gs_loss_kernel(const LossParams p) {
+  using G = GroupT<LN, kLossSplit>;  // two threads per lane, as in the iteration kernel
+  using L = FieldLayout<LN, LN, 1>;
   constexpr int N = G::N;
   constexpr int T = G::T;
+  constexpr int V = G::V;        // elements per thread: t0 + STEP i
+  constexpr int STEP = G::STEP;
+  constexpr int THR = kThreads * kLossSplit;
   constexpr int LOGT = LN - 5;
   constexpr int NG = kThreads / T;
   constexpr int W = L::W;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Shared sh;
   const int b = blockIdx.x;
-  const int gidx = threadIdx.x >> LOGT;
+  const int o = lane_of<kLossSplit>();  // this thread's lane of the block
+  const int gidx = o >> LOGT;
   G grp;
-  grp.t = threadIdx.x & (T - 1);
-  grp.bar_id = 1 + gidx;
+  grp.t = o & (T - 1);
+  grp.c = lane_part<kLossSplit>();
+  grp.bar_id = 1 + (kLossSplit == 1 ? gidx : o / G::TT);
   grp.sm = reinterpret_cast<float2*>(smem) + gidx * G::SMEM;
+  grp.sx = reinterpret_cast<float2*>(smem + kSplitSmemOffset) + (o / G::TT) * G::SPLIT + (o & (G::TT - 1));
   grp.tw = p.tw;
-  const int t = grp.t;
-  StageTw<LN> stw;
-  stw.load(p.tw, t);
+  const int t0 = grp.first();
+  StageTw<LN, kLossSplit> stw;
+  stw.load(p.tw, grp.t, grp.c);
   float* its = reinterpret_cast<float*>(smem + kAmpSmemOffset);
   float2* blk = reinterpret_cast<float2*>(smem + kBlockSmemOffset);
   unsigned target = 0;
@@ -121,10 +127,10 @@ __global__ void __launch_bounds__(kThreads, 1) gs_loss_kernel(const LossParams p
     float max_i = 0.f;
     const float* Ib = p.I + static_cast<size_t>(r0) * N;
     const int cnt = (r1 - r0) * N;
-    for (int e0 = threadIdx.x; e0 < cnt; e0 += 8 * kThreads) {
+    for (int e0 = threadIdx.x; e0 < cnt; e0 += 8 * THR) {
       float xs[8];  // eight loads in flight before they are used
 #pragma unroll
-      for (int u = 0; u < 8; ++u) xs[u] = (e0 + u * kThreads < cnt) ? Ib[e0 + u * kThreads] : 0.f;
+      for (int u = 0; u < 8; ++u) xs[u] = (e0 + u * THR < cnt) ? Ib[e0 + u * THR] : 0.f;
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         bad |= !(fabsf(xs[u]) <= FLT_MAX);
@@ -141,7 +147,7 @@ __global__ void __launch_bounds__(kThreads, 1) gs_loss_kernel(const LossParams p
     __syncthreads();
     if (threadIdx.x == 0) {
       double bmax = 0.0;
-      for (int w = 0; w < kThreads / 32; ++w) bmax = fmax(bmax, sh.red[w]);
+      for (int w = 0; w < THR / 32; ++w) bmax = fmax(bmax, sh.red[w]);
       const int G = gridDim.x;
       p.partials[kRowFlag * G + b] = any_bad ? __longlong_as_double(0x7ff8000000000000ll) : 0.0;
       p.partials[kRowSumI * G + b] = bsum;
@@ -154,14 +160,14 @@ __global__ void __launch_bounds__(kThreads, 1) gs_loss_kernel(const LossParams p
     float* tb = reinterpret_cast<float*>(blk);  // [N][W + 1]
     for (int cb = lo; cb < hi; ++cb) {
       __syncthreads();
-      for (int e = threadIdx.x; e < N * W; e += kThreads) {
+      for (int e = threadIdx.x; e < N * W; e += THR) {
         const int k = e & (W - 1);
         const int y = e >> L::LW;
         cp_async4(tb + y * (W + 1) + k, p.I + static_cast<size_t>(y) * N + cb * W + k);
       }
       cp_async_wait_all();
       __syncthreads();
-      for (int e = threadIdx.x; e < N * W; e += kThreads) {
+      for (int e = threadIdx.x; e < N * W; e += THR) {
         const int k = e >> LN;
         const int y = e & (N - 1);
         p.IT[static_cast<size_t>(cb * W + k) * N + y] = tb[y * (W + 1) + k];
@@ -196,35 +202,36 @@ __global__ void __launch_bounds__(kThreads, 1) gs_loss_kernel(const LossParams p
       const int idx = base + gidx;
       const bool valid = idx < hi;
       const int ridx = valid ? idx : base;
-      float2 v[32];
-      const float* ph = p.phi + static_cast<size_t>(ridx) * N + t;
-      const float* pp = p.p_slm ? p.p_slm + static_cast<size_t>(ridx) * N + t : nullptr;
-      float2* su = grp.sm + t;
+      float2 v[V];
+      const float* ph = p.phi + static_cast<size_t>(ridx) * N + t0;
+      const float* pp = p.p_slm ? p.p_slm + static_cast<size_t>(ridx) * N + t0 : nullptr;
+      float2* su = grp.sm + t0;
+      grp.sync();  // the previous round's transform has read the buffer
       // phi (and p) by cp.async, all loads in flight, then a rolled loop
 #pragma unroll
-      for (int i = 0; i < 32; ++i) cp_async4(&su[T * i].x, ph + T * i);
+      for (int i = 0; i < V; ++i) cp_async4(&su[STEP * i].x, ph + STEP * i);
       if (pp) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) cp_async4(&su[T * i].y, pp + T * i);
+        for (int i = 0; i < V; ++i) cp_async4(&su[STEP * i].y, pp + STEP * i);
       }
       cp_async_wait_all();
       // four copies of sincosf: independent work for the scheduler, while
       // the code stays small (instruction fetch is this kernel's top stall)
 #pragma unroll 4
-      for (int i = 0; i < 32; ++i) {
+      for (int i = 0; i < V; ++i) {
         float s, c;
-        const float2 fa = su[T * i];
+        const float2 fa = su[STEP * i];
         sincosf(fa.x, &s, &c);
         const float a = pp ? fa.y : 1.f;
-        su[T * i] = make_float2(a * c, a * s);
+        su[STEP * i] = make_float2(a * c, a * s);
       }
 #pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = su[T * i];
+      for (int i = 0; i < V; ++i) v[i] = su[STEP * i];
       grp.sync();
       group_fft<LN>(v, grp, stw);
       if (valid) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) p.B[L::off(idx, t + T * i)] = v[i];
+        for (int i = 0; i < V; ++i) p.B[L::off(idx, t0 + STEP * i)] = v[i];
       }
     }
   }
@@ -278,7 +285,7 @@ __global__ void __launch_bounds__(kThreads, 1) gs_loss_kernel(const LossParams p
       const int lo = split(b, gridDim.x, L::NBLK);
       const int hi = split(b + 1, gridDim.x, L::NBLK);
       const bool gact = gidx < W;
-      const bool wact = ((threadIdx.x & ~31) >> LOGT) < W;
+      const bool wact = ((o & ~31) >> LOGT) < W;
       const int gq = gact ? gidx : 0;
       for (int cb = lo; cb < hi; ++cb) {
         __syncthreads();
@@ -299,29 +306,30 @@ __global__ void __launch_bounds__(kThreads, 1) gs_loss_kernel(const LossParams p
           sh.pending = 0;
         }
         if (wact) {
-          float2 v[32];
+          float2 v[V];
 #pragma unroll
-          for (int i = 0; i < 32; ++i) v[i] = blk[L::boff(t + T * i, gq)];
+          for (int i = 0; i < V; ++i) v[i] = blk[L::boff(t0 + STEP * i, gq)];
           group_fft<LN>(v, grp, stw);
-          const float* icol = its + gq * N + t;
-          float* sa2 = reinterpret_cast<float*>(grp.sm) + t;  // |y|^2 for the physical error
+          const float* icol = its + gq * N + t0;
+          float* sa2 = reinterpret_cast<float*>(grp.sm) + t0;  // |y|^2 for the physical error
+          if (want_phys) grp.sync();  // the transform has read the buffer
           float part = 0.f;
 #pragma unroll
-          for (int i = 0; i < 32; ++i) {
+          for (int i = 0; i < V; ++i) {
             const float2 y = v[i];
-            const float a2 = y.x * y.x + y.y * y.y;
-            const float r = a2 * p.inv_n - icol[T * i];
+            const float a2 = norm2(y.x, y.y);
+            const float r = fmaf(a2, p.inv_n, -icol[STEP * i]);
             part = fmaf(r, r, part);
-            if (want_phys) sa2[T * i] = a2;
+            if (want_phys) sa2[STEP * i] = a2;
             v[i] = make_float2(r * y.y, r * y.x);  // swapped: the next forward DFT acts as the inverse
           }
           if (gact) acc += part;
           if (want_phys) {  // Eq. (phys-error), once per call: a rolled loop
             float el = 0.f, ed = 0.f;
 #pragma unroll 1
-            for (int i = 0; i < 32; ++i) {
-              const float ir = sa2[T * i] * ir_scale;  // reconstructed intensity
-              const float iv = icol[T * i];
+            for (int i = 0; i < V; ++i) {
+              const float ir = sa2[STEP * i] * ir_scale;  // reconstructed intensity
+              const float iv = icol[STEP * i];
               if (iv > 0.f) {
                 const float it = iv * it_scale;
                 const float rel = fabsf(it - ir) / it;
@@ -340,7 +348,7 @@ __global__ void __launch_bounds__(kThreads, 1) gs_loss_kernel(const LossParams p
             group_fft<LN>(v, grp, stw);
             if (gact) {
 #pragma unroll
-              for (int i = 0; i < 32; ++i) blk[L::boff(t + T * i, gidx)] = v[i];
+              for (int i = 0; i < V; ++i) blk[L::boff(t0 + STEP * i, gidx)] = v[i];
             }
           }
         }
@@ -414,32 +422,32 @@ __global__ void __launch_bounds__(kThreads, 1) gs_loss_kernel(const LossParams p
         const int idx = base + gidx;
         const bool valid = idx < hi;
         const int ridx = valid ? idx : base;
-        float2 v[32];
+        float2 v[V];
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = p.B[L::off(ridx, t + T * i)];
+        for (int i = 0; i < V; ++i) v[i] = p.B[L::off(ridx, t0 + STEP * i)];
         // phi (and p) of this row by cp.async into the field staging buffer
         // (free in this pass), in flight behind the transform
         float* sph = reinterpret_cast<float*>(blk) + threadIdx.x;
-        float* spp = sph + 32 * kThreads;
+        float* spp = sph + V * THR;
         // the fused update with p = 1: the row's moments too, into the laser
         // amplitude's buffer and the staged target's (free in this pass)
         float* const smm = (adam && !p.p_slm) ? spp : nullptr;
         float* const smv = (adam && !p.p_slm) ? its + threadIdx.x : nullptr;
         {
-          const size_t r0 = static_cast<size_t>(ridx) * N + t;
+          const size_t r0 = static_cast<size_t>(ridx) * N + t0;
           const float* ph = p.phi + r0;
 #pragma unroll
-          for (int i = 0; i < 32; ++i) cp_async4(sph + kThreads * i, ph + T * i);
+          for (int i = 0; i < V; ++i) cp_async4(sph + THR * i, ph + STEP * i);
           if (p.p_slm) {
             const float* pp = p.p_slm + r0;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) cp_async4(spp + kThreads * i, pp + T * i);
+            for (int i = 0; i < V; ++i) cp_async4(spp + THR * i, pp + STEP * i);
           }
           if (smm != nullptr) {
 #pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              cp_async4(smm + kThreads * i, p.m + r0 + T * i);
-              cp_async4(smv + kThreads * i, p.v + r0 + T * i);
+            for (int i = 0; i < V; ++i) {
+              cp_async4(smm + THR * i, p.m + r0 + STEP * i);
+              cp_async4(smv + THR * i, p.v + r0 + STEP * i);
             }
           }
         }
@@ -451,52 +459,53 @@ __global__ void __launch_bounds__(kThreads, 1) gs_loss_kernel(const LossParams p
           if (h == 1) {
             if (valid) {
 #pragma unroll
-              for (int i = 0; i < 32; ++i) p.B[L::off(idx, t + T * i)] = v[i];
+              for (int i = 0; i < V; ++i) p.B[L::off(idx, t0 + STEP * i)] = v[i];
             }
             break;
           }
           // Im(conj(x) z) = x.re z.im - x.im z.re, with z = (v.y, v.x) / N
-          float2* su = grp.sm + t;
+          float2* su = grp.sm + t0;
+          grp.sync();  // the transform has read the buffer
 #pragma unroll
-          for (int i = 0; i < 32; ++i) su[T * i] = v[i];
+          for (int i = 0; i < V; ++i) su[STEP * i] = v[i];
           cp_async_wait_all();
           if (valid && !adam) {
-            float* gr = p.grad + static_cast<size_t>(idx) * N + t;
+            float* gr = p.grad + static_cast<size_t>(idx) * N + t0;
 #pragma unroll 4
-            for (int i = 0; i < 32; ++i) {
+            for (int i = 0; i < V; ++i) {
               float s, c;
-              sincosf(sph[kThreads * i], &s, &c);
-              const float a = p.p_slm ? spp[kThreads * i] : 1.f;  // x = p exp(i phi)
-              const float2 w = su[T * i];
-              gr[T * i] = scale * a * (c * w.x - s * w.y);
+              sincosf(sph[THR * i], &s, &c);
+              const float a = p.p_slm ? spp[THR * i] : 1.f;  // x = p exp(i phi)
+              const float2 w = su[STEP * i];
+              gr[STEP * i] = scale * a * fmaf(c, w.x, -(s * w.y));
             }
           } else if (valid) {
-            const size_t e0 = static_cast<size_t>(idx) * N + t;
+            const size_t e0 = static_cast<size_t>(idx) * N + t0;
 #pragma unroll 4
-            for (int i = 0; i < 32; ++i) {
+            for (int i = 0; i < V; ++i) {
               float s, c;
-              sincosf(sph[kThreads * i], &s, &c);
-              const float a = p.p_slm ? spp[kThreads * i] : 1.f;
-              const float2 w = su[T * i];
-              const float g = scale * a * (c * w.x - s * w.y);
-              const size_t e = e0 + T * i;
-              const float m0 = smm ? smm[kThreads * i] : p.m[e];
-              const float v0 = smv ? smv[kThreads * i] : p.v[e];
+              sincosf(sph[THR * i], &s, &c);
+              const float a = p.p_slm ? spp[THR * i] : 1.f;
+              const float2 w = su[STEP * i];
+              const float g = scale * a * fmaf(c, w.x, -(s * w.y));
+              const size_t e = e0 + STEP * i;
+              const float m0 = smm ? smm[THR * i] : p.m[e];
+              const float v0 = smv ? smv[THR * i] : p.v[e];
               const float mi = fmaf(p.beta1, m0, (1.f - p.beta1) * g);
               const float vi = fmaf(p.beta2, v0, (1.f - p.beta2) * g * g);
               p.m[e] = mi;
               p.v[e] = vi;
-              const float ph = sph[kThreads * i] - adam_step * mi / (sqrtf(vi) * adam_rb2 + p.eps);
+              const float ph = sph[THR * i] - adam_step * mi / fmaf(sqrtf(vi), adam_rb2, p.eps);
               p.phase[e] = ph;
               if (fuse) {  // x = p exp(i phi) of the next step, in place of w
                 sincosf(ph, &s, &c);
-                su[T * i] = make_float2(a * c, a * s);
+                su[STEP * i] = make_float2(a * c, a * s);
               }
             }
           }
           if (fuse) {  // a group with no row of its own transforms what it holds and stores nothing
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = su[T * i];
+            for (int i = 0; i < V; ++i) v[i] = su[STEP * i];
             grp.sync();
           }
         }

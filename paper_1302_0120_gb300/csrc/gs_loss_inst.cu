@@ -28,11 +28,11 @@ static const void* loss_kernel_for(int logn, int mode) {
 cudaError_t launch_loss(const LossParams& p, int grid, cudaStream_t s) {
   const void* k = loss_kernel_for(p.logn, p.mode);
   if (k == nullptr) return cudaErrorInvalidValue;
-  const size_t smem = iteration_smem_bytes(p.n, p.n);
+  const size_t smem = kGroupSmemBytes + 8192 * 4 + 8192 * 8 + (kLossSplit > 1 ? kSplitSmemBytes : 0);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kThreads * kLossSplit, smem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -40,7 +40,7 @@ cudaError_t launch_loss(const LossParams& p, int grid, cudaStream_t s) {
   if (grid > per_sm * sms) grid = per_sm * sms;
   if (grid < 1) grid = 1;
   void* args[] = {const_cast<LossParams*>(&p)};
-  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads), args, smem, s);
+  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kThreads * kLossSplit), args, smem, s);
 }
 
 }  // namespace gsk

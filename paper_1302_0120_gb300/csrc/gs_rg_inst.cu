@@ -19,7 +19,7 @@ __global__ void __launch_bounds__(kThreads, 1) gs_iterate_rg(const Params p) {
   __shared__ Shared sh;
   if (*reinterpret_cast<volatile int*>(p.abort_flag) != 0) return;  // an earlier chunk failed
   const StageTw<5> none{};
-  iterate_class<NX, NY, false>(p, sh, smem, none, NoTc{});
+  iterate_class<NX, NY, false>(p, sh, smem, none, NoTc<1>{});
 }
 
 template <>

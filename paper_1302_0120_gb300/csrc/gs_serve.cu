@@ -56,7 +56,7 @@ int ensure_running(gs_server* s) {
   __atomic_store_n(&s->table->running, 1, __ATOMIC_SEQ_CST);
   void* args[] = {&s->sp};
   if (cudaMemsetAsync(s->sp.base.bar, 0, sizeof(unsigned), s->stream) != cudaSuccess ||
-      cudaLaunchCooperativeKernel(serve_kernel(), dim3(s->grid), dim3(gsk::kThreads), args, s->smem, s->stream) !=
+      cudaLaunchCooperativeKernel(serve_kernel(), dim3(s->grid), dim3(gsk::kThreads * gsk::kMixedSplit), args, s->smem, s->stream) !=
           cudaSuccess ||
       cudaEventRecord(s->ev, s->stream) != cudaSuccess) {
     cudaGetLastError();
@@ -84,12 +84,12 @@ int gs_serve_create(gs_server** out, int max_n, int slots, int grid, void* strea
   s->L = L;
   s->slots = slots;
   s->stream = static_cast<cudaStream_t>(stream);
-  s->smem = static_cast<size_t>(gsk::kGroupSmemBytes) + 8192 * 4 + 8192 * 8;
+  s->smem = static_cast<size_t>(gsk::kGroupSmemBytes) + 8192 * 4 + 8192 * 8 + (gsk::kMixedSplit > 1 ? gsk::kSplitSmemBytes : 0);
   int dev = 0, sms = 0, per_sm = 0;
   const void* k = serve_kernel();
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(s->smem)) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, gsk::kThreads, s->smem) != cudaSuccess || per_sm < 1) {
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, gsk::kThreads * gsk::kMixedSplit, s->smem) != cudaSuccess || per_sm < 1) {
     cudaGetLastError();
     delete s;
     return GS_ECUDA;

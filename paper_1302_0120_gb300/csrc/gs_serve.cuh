@@ -296,7 +296,7 @@ __device__ __forceinline__ void serve_a0_partial(const Params& p, double* part, 
   const int cnt = (r1 - r0) * p.nx;
   double acc = 0.0;
   bool bad = false;
-  for (int e = threadIdx.x; e < cnt; e += kThreads) {
+  for (int e = threadIdx.x; e < cnt; e += kThreads * kMixedSplit) {
     const float x = I[e];
     bad |= !(x >= 0.f && x <= FLT_MAX);
     acc += static_cast<double>(x);
@@ -310,21 +310,21 @@ __device__ __forceinline__ void serve_a0_partial(const Params& p, double* part, 
 // dispatched on the slot's grid.
 __device__ __forceinline__ float serve_run_pass(const Params& p, int kind, bool last, int lo, int hi,
                                                 unsigned char* smem, Shared& sh, unsigned& mphase) {
-  const NoTc tcf{};
+  const NoTc<kMixedSplit, false> tcf{};  // the request table takes the second staging buffer's place
   if (p.logny == 8) {
-    const StageTw<8> none{};
+    const StageTw<8, kMixedSplit> none{};
     return run_pass<8, 8, 8, false>(p, 0, kind, last, lo, hi, smem, sh, mphase, none, tcf);
   }
   if (p.logny == 9) {
-    const StageTw<9> none{};
+    const StageTw<9, kMixedSplit> none{};
     return run_pass<9, 9, 9, false>(p, 0, kind, last, lo, hi, smem, sh, mphase, none, tcf);
   }
-  const StageTw<10> none{};
+  const StageTw<10, kMixedSplit> none{};
   return run_pass<10, 10, 10, false>(p, 0, kind, last, lo, hi, smem, sh, mphase, none, tcf);
 }
 
 // The persistent serving kernel.
-__global__ void __launch_bounds__(kThreads, 1) gs_serve(const ServeParams sp) {
+__global__ void __launch_bounds__(kThreads * kMixedSplit, 1) gs_serve(const ServeParams sp) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Shared sh;
   __shared__ ServePlan plan;
@@ -348,7 +348,7 @@ __global__ void __launch_bounds__(kThreads, 1) gs_serve(const ServeParams sp) {
     {
       const int* src = reinterpret_cast<const int*>(&sp.st->plan[t & 1]);
       int* dst = reinterpret_cast<int*>(&plan);
-      for (int e = threadIdx.x; e < static_cast<int>(sizeof(ServePlan) / 4); e += kThreads) dst[e] = __ldcg(src + e);
+      for (int e = threadIdx.x; e < static_cast<int>(sizeof(ServePlan) / 4); e += kThreads * kMixedSplit) dst[e] = __ldcg(src + e);
     }
     __syncthreads();
     {
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, 1) gs_serve(const ServeParams sp) {
       constexpr int kW = static_cast<int>(sizeof(Params) / 4);
       for (int s = 0; s < S; ++s)
         if (t == 0 || plan.col[s] == kColA0)
-          for (int e = threadIdx.x; e < kW; e += kThreads) pd[s * kW + e] = __ldcg(ps + s * kW + e);
+          for (int e = threadIdx.x; e < kW; e += kThreads * kMixedSplit) pd[s * kW + e] = __ldcg(ps + s * kW + e);
     }
     __syncthreads();
     // finish the previous tick: its row gaps, and the requests it completed
@@ -406,8 +406,7 @@ __global__ void __launch_bounds__(kThreads, 1) gs_serve(const ServeParams sp) {
           sh.bad[s] = bad ? 1 : 0;
           sh.scale[s] = bad ? 0.f : static_cast<float>(sqrt(static_cast<double>(prm[s].nx) * prm[s].ny / total));
           // the slot's amplitude is rebuilt: no column block of it stays resident
-          sh.m_block = nullptr;
-          sh.m_slot[0] = sh.m_slot[1] = nullptr;
+          for (int k = 0; k < kMaxSlots; ++k) sh.m_slot[k] = nullptr;
         }
       }
       __syncthreads();
