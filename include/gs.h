@@ -29,8 +29,8 @@
  *   - nx and ny are powers of two in [8, 4096] or 5-smooth numbers
  *     (2^a 3^b 5^c, such as the 800 x 600 SLM of Sec. V) in [8, 1536].
  *     Grids with both sides powers of two of at least 32 run on the
- *     register-resident kernels (one block per mask when the grid has at
- *     most 8192 pixels, see gs_run); every other grid on the general kernel.
+ *     register-resident kernels (one cluster per mask when the grid has at
+ *     most 32768 pixels, see gs_run); every other grid on the general kernel.
  *
  * Memory and ordering:
  *   - Pointers named "device" are CUDA device pointers owned by the caller;
@@ -154,8 +154,10 @@ int gs_create_batched(gs_ctx** out, int nx, int ny, int max_batch, unsigned flag
  * reported by gs_status; on GS_ENUMERIC the phase output is left untouched and
  * residuals are set to NaN.
  * Execution: one persistent cooperative launch per 128 iterations; grids of
- * power-of-two sides >= 32 with at most 8192 pixels (64 x 64, 32 x 256, ...)
- * instead run the whole run in one launch of one block per mask with the
+ * power-of-two sides 32 ... 256 with at most 32768 pixels (64 x 64, 32 x 256,
+ * 128 x 256, ...) instead run the whole run in one launch of one cluster of at
+ * most 8 blocks per mask (batches of more than 8192 pixels per mask only while
+ * every mask has its cluster at once) with the
  * field in shared memory (same iterates bit for bit), unless gs_set_grid
  * fixed a grid, or the target start, a laser amplitude or pass timestamps
  * are in use.
@@ -506,7 +508,7 @@ int gs_adam_step(float* phase, const float* grad, float* m, float* v, long long 
  * context workspace, and calls no cudaMalloc, cudaFree or allocating routine.
  * It always runs the persistent kernel with gs_run's automatic grid (one
  * block per 4096 pixels, small grids up to 32 blocks), also for the grids of
- * at most 8192 pixels that gs_run hands to its one-block-per-mask kernel:
+ * at most 32768 pixels that gs_run hands to its one-cluster-per-mask kernel:
  * the iterates are the same, such a small grid only runs slower here.
  *   nx, ny          powers of two in [32, 4096] with nx * ny <= 262144
  *                   (512 x 512): the static scratch holds one such grid.

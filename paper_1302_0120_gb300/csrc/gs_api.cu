@@ -196,6 +196,7 @@ struct gs_ctx {
   int blocks_per_sm = 0;
   int grid_override = 0;
   int tc_mode = 0;               // gsk::TcMode of the iteration kernel
+  int small_clusters[gsk::kSmallMaxLogC + 1] = {};  // small grids: clusters of 2^lc blocks that run at once
   bool loss_prepared = false;    // the workspace holds a target staged by gs_loss_prepare
   const float* p_slm = nullptr;  // caller-owned SLM amplitude, or null (p = 1)
   unsigned extra_arrivals = 0;
@@ -282,6 +283,20 @@ int check_guards(const unsigned char* ws, const Layout& L) {
   return GS_OK;
 }
 
+// log2 of the blocks per mask of a small-grid run: the most for which every
+// block of the batch has an SM (64 masks of 64 x 64 x 20 iterations: 110 us
+// with two blocks each, 125 with four that share SMs). Without any, the fewest
+// blocks,
+// where shared memory has room for the grid on one or two SMs (at most 8192
+// pixels); larger grids then run on the persistent kernel (-1), which shares
+// the device between the masks.
+int small_logc(const gs_ctx* c, int batch) {
+  for (int lc = gsk::kSmallMaxLogC; lc >= 0; --lc)
+    if (c->small_clusters[lc] >= batch && (batch << lc) <= c->num_sms) return lc;
+  const int lc = gsk::small_min_logc(c->nx, c->ny);
+  return lc <= 1 && c->small_clusters[lc] > 0 ? lc : -1;
+}
+
 bool on_general(const gs_ctx* c) { return !c->mixed && gsk::uses_general(c->nx, c->ny) && !gsk::uses_rg(c->nx, c->ny); }
 
 // Blocks of a run of `masks` masks iterated together: a pass splits the rows
@@ -362,7 +377,7 @@ int gs_create_batched(gs_ctx** out, int nx, int ny, int max_batch, unsigned flag
   if (cudaGetDevice(&c->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess ||
       gsk::iteration_occupancy(nx, ny, &c->blocks_per_sm, tc_mode) != cudaSuccess || c->blocks_per_sm < 1 ||
-      (gsk::small_grid(nx, ny) && gsk::small_prepare(nx, ny) != cudaSuccess)) {
+      (gsk::small_grid(nx, ny) && gsk::small_prepare(nx, ny, c->small_clusters) != cudaSuccess)) {
     cudaGetLastError();
     delete c;
     return GS_ECUDA;
@@ -402,12 +417,13 @@ int gs_run_batched(gs_ctx* c, int batch, const float* target_intensity, const fl
   if (c == nullptr || c->mixed || target_intensity == nullptr || (phase_in == nullptr && !from_target) ||
       phase_out == nullptr || iters < 0 || batch < 1 || batch > c->max_batch)
     return GS_EINVAL;
-  // Small grids run one block per mask with the field in shared memory,
+  // Small grids run one cluster per mask with the field in shared memory,
   // unless a fixed grid, a variant the small kernel does not implement (the
   // target start, a laser amplitude, tensor cores) or a diagnostic (pass
   // timestamps, the barrier test hook) asks for the persistent kernel.
   const bool small = gsk::small_grid(c->nx, c->ny) && c->grid_override == 0 && !from_target &&
-                     c->p_slm == nullptr && !(c->flags & GS_TENSOR_CORE) && !c->trace && c->extra_arrivals == 0;
+                     c->p_slm == nullptr && !(c->flags & GS_TENSOR_CORE) && !c->trace && c->extra_arrivals == 0 &&
+                     small_logc(c, batch) >= 0;
   const int group = group_size(c, static_cast<long long>(c->nx) * c->ny, batch);
   const int grid = choose_grid(c, group);
   c->loss_prepared = false;  // the run's amplitude overwrites a staged loss target
@@ -458,6 +474,7 @@ int gs_run_batched(gs_ctx* c, int batch, const float* target_intensity, const fl
     p.it0 = 0;
     p.it1 = iters;
     p.do_init = p.do_final = 1;
+    p.small_logc = small_logc(c, batch);
     if (gsk::launch_small(p, c->stream) != cudaSuccess) {
       cudaGetLastError();
       return GS_ECUDA;

@@ -168,25 +168,30 @@ __host__ __device__ __forceinline__ void dft(float2 (&a)[R]) {
   for (int i = 0; i < R; ++i) a[i] = t[i];
 }
 
+// Values per lane of a team's split-exchange buffer.
+__host__ __device__ constexpr int split_values(int S) { return S == 2 ? 16 : 32; }
+
 // Per-group state of a distributed transform of length N = 2^LOGN. The
 // geometry is a compile-time constant so that every register and
 // shared-memory index folds to an immediate offset.
 //
 // The line is laid out over T = N/32 lanes; lane t owns the 32 elements
-// x[t + T i'], i' = 0..31. S = 1: one thread holds all of them. S = 2: two
-// threads share a lane, thread c = 0, 1 with the 16 elements of parity
-// i' = 2 i + c; the two sit in the same lane of two neighbouring warps, so
-// that c is uniform over a warp. The transform evaluates the same butterflies
-// on the same operands in either form (the results are equal bit for bit):
-// the radix-2 decimation-in-time stages of a 32-point DFT work on the even and
-// the odd inputs separately until the last one, which pairs the two threads.
+// x[t + T i'], i' = 0..31. S = 1: one thread holds all of them. S = 2 or 4:
+// S threads share a lane, thread c with the elements i' = S i + c; they sit in
+// the same lane of neighbouring warps, so that c is uniform over a warp. The
+// transform evaluates the same butterflies on the same operands in each form
+// (the results are equal bit for bit): the radix-2 decimation-in-time stages
+// of a 32-point DFT work on the inputs of equal i' mod S separately until the
+// last log2 S stages, which combine the threads of a lane (split_last). S = 4
+// serves lengths up to 256.
 //
-// Why S = 2: a lane's two transforms, projection and copies are a chain of
-// some 2600 dependent-issue instructions, which one warp alone on its
-// scheduler runs at 3.3 cycles each (4.1 us of a 5.4 us pass at 256 x 256,
-// 5.8-6.8 of 7-8 us at 1024 x 1024 where a scheduler has two such warps).
-// Two threads per lane halve the chain and double the warps in flight; the
-// price is one more exchange of half the line per 32-point DFT.
+// Why: a lane's two transforms, projection and copies are a chain of some 2600
+// dependent-issue instructions, which one warp alone on its scheduler runs at
+// 3.3 cycles each. More threads per lane shorten the chain and put more warps
+// in flight, at the price of one more exchange per 32-point DFT. Column pass
+// of one mask, from loaded to stored: 256 x 256 6000 cycles with S = 1, 3400
+// with S = 2; 512 x 512 6668 and 4720; 1024 x 1024, where a scheduler has two
+// warps of S = 1, 8389 and 9131.
 template <int LOGN, int S = 1>
 struct GroupT {
   static constexpr int N = 1 << LOGN;
@@ -194,13 +199,13 @@ struct GroupT {
   static constexpr int V = 32 / S;         // elements per thread
   static constexpr int SMEM = N + N / 32;  // padded exchange buffer (complex)
   static constexpr int TT = T > 32 ? T : 32;  // lanes that synchronise together (a team)
-  static constexpr int SPLIT = 16 * TT;    // a team's split-exchange buffer (complex), S = 2
-  static_assert(S == 1 || S == 2, "one or two threads per lane");
+  static constexpr int SPLIT = split_values(S) * TT;  // a team's split-exchange buffer (complex), S > 1
+  static_assert(S == 1 || S == 2 || (S == 4 && LOGN <= 8), "threads per lane");
   int t;                                   // lane in the line, 0..T-1
-  int c;                                   // parity of this thread's elements (0 if S = 1)
-  int bar_id;                              // named barrier id (S = 1: T > 32; S = 2: the team's)
+  int c;                                   // residue of this thread's elements i' mod S
+  int bar_id;                              // named barrier id (S = 1: T > 32; S > 1: the team's)
   float2* sm;                              // this line's exchange buffer
-  float2* sx;                              // the team's split-exchange buffer at this lane, S = 2
+  float2* sx;                              // the team's split-exchange buffer at this lane, S > 1
   const float2* __restrict__ tw;           // stage twiddle tables (twiddle_offset)
 
   __device__ __forceinline__ void sync() const {
@@ -219,11 +224,11 @@ struct GroupT {
 // the threads of a lane sit in neighbouring warps.
 template <int S>
 __device__ __forceinline__ int lane_of() {
-  return S == 1 ? threadIdx.x : ((threadIdx.x >> 6) << 5) | (threadIdx.x & 31);
+  return S == 1 ? threadIdx.x : ((threadIdx.x / (32 * S)) << 5) | (threadIdx.x & 31);
 }
 template <int S>
 __device__ __forceinline__ int lane_part() {
-  return S == 1 ? 0 : (threadIdx.x >> 5) & 1;
+  return S == 1 ? 0 : (threadIdx.x >> 5) & (S - 1);
 }
 
 // Twiddle tables. For the stage with Ns = 2^NSL and radix R the factors
@@ -290,6 +295,41 @@ __device__ __forceinline__ void split_last(float2 (&v)[16], const G& g) {
   for (int i = 0; i < 16; ++i) v[i] = o[i];
 }
 
+// The last two stages shared by the four threads of a lane (S = 4): v holds the
+// 8-point DFT of the inputs i' = c mod 4, position j = 0..7. The thread forms
+// the outputs k = j + 8 b (b < 4) of its positions j = C and C + 4, that is
+// k = C mod 4, from the four threads' values at j. Decimation in time pairs
+// the inputs of residues 0 and 2 and those of 1 and 3 first (half-span 8), then
+// the two pairs (half-span 16).
+template <int C, int J, class G>
+__device__ __forceinline__ void split_quad(const float2 (&v)[8], float2 (&o)[8], const G& g) {
+  float2 u[4];  // by residue
+#pragma unroll
+  for (int c = 0; c < 4; ++c) u[c] = c == C ? v[J] : g.sx[(8 * c + J) * G::TT];
+  bfly<2 * J>(u[0], u[2]);  // positions J, J + 8 of the even inputs
+  bfly<2 * J>(u[1], u[3]);  // ... of the odd ones
+  bfly<J>(u[0], u[1]);      // outputs J, J + 16
+  bfly<J + 8>(u[2], u[3]);  // outputs J + 8, J + 24
+  constexpr int I = J / 4;  // register of output k: (k - C) / 4
+  o[I] = u[0];
+  o[I + 2] = u[2];
+  o[I + 4] = u[1];
+  o[I + 6] = u[3];
+}
+
+template <int C, class G>
+__device__ __forceinline__ void split_last(float2 (&v)[8], const G& g) {
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+    if (j % 4 != C) g.sx[(8 * C + j) * G::TT] = v[j];
+  g.sync();
+  float2 o[8];
+  split_quad<C, C>(v, o, g);
+  split_quad<C, C + 4>(v, o, g);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = o[i];
+}
+
 // 32-point DFT over the elements i' of a lane.
 template <class G>
 __device__ __forceinline__ void dft32(float2 (&v)[G::V], const G& g) {
@@ -297,6 +337,13 @@ __device__ __forceinline__ void dft32(float2 (&v)[G::V], const G& g) {
   if constexpr (G::V == 16) {
     if (g.c == 0) split_last<0>(v, g);
     else split_last<1>(v, g);
+  } else if constexpr (G::V == 8) {
+    switch (g.c) {
+      case 0: split_last<0>(v, g); break;
+      case 1: split_last<1>(v, g); break;
+      case 2: split_last<2>(v, g); break;
+      default: split_last<3>(v, g); break;
+    }
   }
 }
 
@@ -340,7 +387,7 @@ __device__ __forceinline__ void stage_c(float2 (&v)[32 / S], const GroupT<LOGN, 
 // m goes to (t / Ns) 32 Ns + (t mod Ns) + m Ns; then every thread reads back
 // its elements x[t + T i']. Index i of the padded buffer lives at i + i/32.
 //
-// S = 2 needs no second barrier: the buffer is next written behind the
+// S > 1 needs no second barrier: the buffer is next written behind the
 // barrier of the next split exchange, which every thread reaches after its
 // reads here.
 template <int LOGN, int NSL, int S>
@@ -370,10 +417,11 @@ __device__ __forceinline__ void exchange(float2 (&v)[32 / S], const GroupT<LOGN,
 #pragma unroll
     for (int i = 0; i < V; ++i) v[i] = r[i * T + ((i * T) >> 5)];
   } else {
-    // (2 i T + c T + t) >> 5 = (2 i T) >> 5: c T + t < 2 T divides 32
+    // (S i T + c T + t) >> 5 = (S i T) >> 5, since c T + t < S T divides 32
+    static_assert(S * T <= 32, "a thread's elements are whole rows of the padding apart");
     const float2* r = g.sm + g.t + c * T;
 #pragma unroll
-    for (int i = 0; i < V; ++i) v[i] = r[2 * i * T + ((2 * i * T) >> 5)];
+    for (int i = 0; i < V; ++i) v[i] = r[S * i * T + ((S * i * T) >> 5)];
   }
   if constexpr (S == 1) g.sync();
 }
@@ -391,12 +439,12 @@ __device__ __forceinline__ void fft_from(float2 (&v)[32 / S], const GroupT<LOGN,
 
 // Forward unnormalised DFT of length N over the group: the thread's registers
 // hold x[first() + STEP i] on entry and X[first() + STEP i] on exit. Every
-// thread of the team must call it. S = 2: other uses of the exchange buffer
+// thread of the team must call it. S > 1: other uses of the exchange buffer
 // after it start with a sync() (other threads may still be reading).
 template <int LOGN, int S>
 __device__ __forceinline__ void group_fft(float2 (&v)[32 / S], const GroupT<LOGN, S>& g, const StageTw<LOGN, S>& sw) {
   // lengths that end in a 32-point DFT: its split exchange may still be read
-  if constexpr (S == 2 && LOGN % 5 == 0) g.sync();
+  if constexpr (S > 1 && LOGN % 5 == 0) g.sync();
   fft_from<LOGN, 0, S>(v, g, sw);
 }
 

@@ -83,6 +83,7 @@ struct Params {
   unsigned planx, plany;
   int nstx, nsty;
   int gen_teams, gen_team_log;  // teams of a block, log2 of a team's threads
+  int small_logc;      // log2 of the blocks per mask of the small-grid kernel
 };
 
 // Three size classes in one launch: square grids 256, 512 and 1024
@@ -93,12 +94,26 @@ struct MixedParams {
   Params cls[3];
 };
 
-// Small grids (power-of-two sides >= 32, at most this many pixels) run one
-// block per mask with the whole field in shared memory (gs_small.cuh).
-constexpr int kSmallMaxPixels = 8192;
+// Small grids (power-of-two sides 32 ... 256, at most this many pixels) run on
+// a cluster of 2^lc blocks per mask with the whole field in their shared
+// memory (gs_small.cuh).
+constexpr int kSmallMaxPixels = 32768;
+constexpr int kSmallMaxLogC = 3;  // 8 blocks, the largest portable cluster
 inline __host__ __device__ bool small_grid(int nx, int ny) {
   const bool px = nx > 0 && (nx & (nx - 1)) == 0, py = ny > 0 && (ny & (ny - 1)) == 0;
-  return px && py && nx >= 32 && ny >= 32 && static_cast<long long>(nx) * ny <= kSmallMaxPixels;
+  return px && py && nx >= 32 && ny >= 32 && nx <= 256 && ny <= 256 && nx * ny <= kSmallMaxPixels;
+}
+// Blocks: at most 4096 pixels each (two fields, the amplitude and the exchange
+// buffers in shared memory), at least 1024 (one warp of lanes).
+inline int small_min_logc(int nx, int ny) {
+  int lc = 0;
+  while ((nx * ny >> lc) > 4096) ++lc;
+  return lc;
+}
+inline int small_max_logc(int nx, int ny) {
+  int lc = 0;
+  while (lc < kSmallMaxLogC && (nx * ny >> lc) > 1024) ++lc;
+  return lc;
 }
 
 // The general kernel serves every grid with a side that is not a power of
@@ -249,9 +264,11 @@ cudaError_t iteration_occupancy(int nx, int ny, int* blocks_per_sm, int tc_mode 
 // The tcgen05 kernel of n x n masks, log2(n) = l in 8..10 (gs_tc5_inst.cu);
 // FP16 or BF16 operands; null for other sizes.
 const void* iterate_kernel_tc5(int l, bool bf16);
-// Small grids (small_grid): allow the kernel its shared memory, and launch
-// one block per mask of p.batch (gs_small_inst.cu).
-cudaError_t small_prepare(int nx, int ny);
+// Small grids (small_grid): allow the kernel its shared memory and find how
+// many clusters of 2^lc blocks run at once (0 where lc does not apply), and
+// launch one cluster of 2^small_logc blocks per mask of p.batch
+// (gs_small_inst.cu).
+cudaError_t small_prepare(int nx, int ny, int clusters[kSmallMaxLogC + 1]);
 cudaError_t launch_small(const Params& p, cudaStream_t s);
 
 }  // namespace gsk

@@ -28,7 +28,7 @@ static const void* loss_kernel_for(int logn, int mode) {
 cudaError_t launch_loss(const LossParams& p, int grid, cudaStream_t s) {
   const void* k = loss_kernel_for(p.logn, p.mode);
   if (k == nullptr) return cudaErrorInvalidValue;
-  const size_t smem = kGroupSmemBytes + 8192 * 4 + 8192 * 8 + (kLossSplit > 1 ? kSplitSmemBytes : 0);
+  const size_t smem = kGroupSmemBytes + 8192 * 4 + 8192 * 8 + lane_smem_bytes(kLossSplit);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   int per_sm = 0;

@@ -1,5 +1,5 @@
 // gs_small_inst.cu -- the small-grid kernels (gs_small.cuh) for every grid of
-// power-of-two sides >= 32 with at most kSmallMaxPixels pixels, and their
+// power-of-two sides 32 ... 256 with at most kSmallMaxPixels pixels, and their
 // host-side launch.
 #include "gs_small.cuh"
 
@@ -7,22 +7,17 @@ namespace gsk {
 
 namespace {
 
-template <int LX, int LY>
-struct SmallKernel {
-  static const void* fn() { return reinterpret_cast<const void*>(&gs_small<LX, LY>); }
-  static constexpr int kThreadsPerBlock = SmallGeom<LX, LY>::NT;
-  static constexpr int kSmem = SmallGeom<LX, LY>::SMEM;
-};
-
 struct SmallEntry {
   const void* fn;
-  int threads;
-  int smem;
+  int (*smem)(int lc);
+  int (*lanes)(int lc);
 };
 
 template <int LX, int LY>
 SmallEntry entry() {
-  return {SmallKernel<LX, LY>::fn(), SmallKernel<LX, LY>::kThreadsPerBlock, SmallKernel<LX, LY>::kSmem};
+  using Gm = SmallGeom<LX, LY>;
+  return {reinterpret_cast<const void*>(&gs_small<LX, LY>), [](int lc) { return Gm::smem(lc); },
+          [](int lc) { return Gm::lanes(lc); }};
 }
 
 int log2_of(int n) {
@@ -41,26 +36,55 @@ bool lookup(int nx, int ny, SmallEntry* e) {
     case 6 * 16 + 5: *e = entry<6, 5>(); return true;
     case 6 * 16 + 6: *e = entry<6, 6>(); return true;
     case 6 * 16 + 7: *e = entry<6, 7>(); return true;
+    case 6 * 16 + 8: *e = entry<6, 8>(); return true;
     case 7 * 16 + 5: *e = entry<7, 5>(); return true;
     case 7 * 16 + 6: *e = entry<7, 6>(); return true;
+    case 7 * 16 + 7: *e = entry<7, 7>(); return true;
+    case 7 * 16 + 8: *e = entry<7, 8>(); return true;
     case 8 * 16 + 5: *e = entry<8, 5>(); return true;
+    case 8 * 16 + 6: *e = entry<8, 6>(); return true;
+    case 8 * 16 + 7: *e = entry<8, 7>(); return true;
     default: return false;
   }
 }
 
+cudaLaunchConfig_t config(const SmallEntry& e, int batch, int lc, cudaLaunchAttribute* attr, cudaStream_t s) {
+  attr->id = cudaLaunchAttributeClusterDimension;
+  attr->val.clusterDim.x = 1u << lc;
+  attr->val.clusterDim.y = attr->val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(static_cast<unsigned>(batch) << lc);
+  cfg.blockDim = dim3(4 * e.lanes(lc));
+  cfg.dynamicSmemBytes = e.smem(lc);
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cfg;
+}
+
 }  // namespace
 
-cudaError_t small_prepare(int nx, int ny) {
+cudaError_t small_prepare(int nx, int ny, int clusters[kSmallMaxLogC + 1]) {
+  for (int lc = 0; lc <= kSmallMaxLogC; ++lc) clusters[lc] = 0;
   SmallEntry e;
   if (!lookup(nx, ny, &e)) return cudaErrorInvalidValue;
-  return cudaFuncSetAttribute(e.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem);
+  const int lo = small_min_logc(nx, ny), hi = small_max_logc(nx, ny);
+  cudaError_t rc = cudaFuncSetAttribute(e.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, e.smem(lo));
+  for (int lc = lo; lc <= hi && rc == cudaSuccess; ++lc) {
+    cudaLaunchAttribute attr;
+    const cudaLaunchConfig_t cfg = config(e, 1, lc, &attr, nullptr);
+    rc = cudaOccupancyMaxActiveClusters(&clusters[lc], e.fn, &cfg);
+  }
+  return rc;
 }
 
 cudaError_t launch_small(const Params& p, cudaStream_t s) {
   SmallEntry e;
   if (!lookup(p.nx, p.ny, &e)) return cudaErrorInvalidValue;
+  cudaLaunchAttribute attr;
+  const cudaLaunchConfig_t cfg = config(e, p.batch, p.small_logc, &attr, s);
   void* args[] = {const_cast<Params*>(&p)};
-  return cudaLaunchKernel(e.fn, dim3(p.batch), dim3(e.threads), args, e.smem, s);
+  return cudaLaunchKernelExC(&cfg, e.fn, args);
 }
 
 }  // namespace gsk
