@@ -74,6 +74,25 @@ static __device__ bool loss_sync(const LossParams& p, unsigned& target, Shared& 
   return sh.flag != 0;
 }
 
+// The target's statistics from the blocks' partials, by one warp in a fixed
+// order (the result in every lane). Every thread adding all of them in turn
+// held up each call by the latency of three FP64 chains over the grid.
+static __device__ void loss_target_stats(const LossParams& p, double& flag, double& sum_i, double& max_i) {
+  const int G = gridDim.x;
+  flag = sum_i = max_i = 0.0;
+  for (int c = threadIdx.x & 31; c < G; c += 32) {
+    flag += p.partials[kRowFlag * G + c];
+    sum_i += p.partials[kRowSumI * G + c];
+    max_i = fmax(max_i, p.partials[kRowMaxI * G + c]);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    flag += __shfl_xor_sync(0xffffffffu, flag, o);
+    sum_i += __shfl_xor_sync(0xffffffffu, sum_i, o);
+    max_i = fmax(max_i, __shfl_xor_sync(0xffffffffu, max_i, o));
+  }
+}
+
 // MODE (LossMode, gs_internal.h) kLossFused: validate and stage the target,
 // then the three passes (one call does everything). kLossPrepare: validate
 // and stage the target only, and reduce its statistics into row kRowStaged.
@@ -177,19 +196,16 @@ __global__ void __launch_bounds__(kThreads * kLossSplit, 1) gs_loss_kernel(const
   if constexpr (MODE == kLossPrepare) {
     // the staged target's statistics, reduced once (FP64, fixed order)
     if (!loss_sync(p, target, sh)) return;
-    if (b == 0 && threadIdx.x == 0) {
-      const int G = gridDim.x;
-      double flag = 0.0, sum_i = 0.0, max_i = 0.0;
-      for (int c = 0; c < G; ++c) {
-        flag += p.partials[kRowFlag * G + c];
-        sum_i += p.partials[kRowSumI * G + c];
-        max_i = fmax(max_i, p.partials[kRowMaxI * G + c]);
+    if (b == 0 && threadIdx.x < 32) {
+      double flag, sum_i, max_i;
+      loss_target_stats(p, flag, sum_i, max_i);
+      if (threadIdx.x == 0) {
+        double* st = p.partials + kRowStaged * kMaxGrid;  // a fixed place: the step may use another grid
+        st[0] = flag;
+        st[1] = sum_i;
+        st[2] = max_i;
+        if (!(flag == 0.0)) atomicCAS(p.status, 0, GS_ENUMERIC);
       }
-      double* st = p.partials + kRowStaged * kMaxGrid;  // a fixed place: the step may use another grid
-      st[0] = flag;
-      st[1] = sum_i;
-      st[2] = max_i;
-      if (!(flag == 0.0)) atomicCAS(p.status, 0, GS_ENUMERIC);
     }
     return;
   }
@@ -241,18 +257,25 @@ __global__ void __launch_bounds__(kThreads * kLossSplit, 1) gs_loss_kernel(const
   float ir_scale = 0.f, it_scale = 0.f;
   {
     double tot = 0.0, sum_i = 0.0, max_i = 0.0;
-    const int G = gridDim.x;
     if constexpr (MODE == kLossStep) {
       const double* st = p.partials + kRowStaged * kMaxGrid;  // written by the prepare launch
       tot = st[0];
       sum_i = st[1];
       max_i = st[2];
     } else {
-      for (int c = 0; c < G; ++c) {
-        tot += p.partials[kRowFlag * G + c];
-        sum_i += p.partials[kRowSumI * G + c];
-        max_i = fmax(max_i, p.partials[kRowMaxI * G + c]);
+      if (threadIdx.x < 32) {
+        loss_target_stats(p, tot, sum_i, max_i);
+        if (threadIdx.x == 0) {
+          sh.red[0] = tot;
+          sh.red[1] = sum_i;
+          sh.red[2] = max_i;
+        }
       }
+      __syncthreads();
+      tot = sh.red[0];
+      sum_i = sh.red[1];
+      max_i = sh.red[2];
+      __syncthreads();  // sh.red is reused
     }
     const double ep = p.p_slm ? *p.energy : static_cast<double>(N) * N;
     if (max_i > 0.0 && ep > 0.0) {

@@ -43,10 +43,13 @@ class LossContext:
         cur = torch.cuda.current_stream(phase.device)
         loss = torch.empty(1, dtype=torch.float64, device=phase.device)
         grad = torch.empty_like(phase) if want_grad else None
-        self.stream.wait_stream(cur)
+        other = cur != self.stream  # the same stream is ordered as it is
+        if other:
+            self.stream.wait_stream(cur)
         rc = B.gs_loss_grad(self.handle, target.data_ptr(), phase.data_ptr(), loss.data_ptr(),
                             grad.data_ptr() if grad is not None else 0)
-        cur.wait_stream(self.stream)
+        if other:
+            cur.wait_stream(self.stream)
         if rc != B.GS_OK:
             raise B.GSError(rc, "gs_loss_grad")
         return loss, grad
@@ -73,10 +76,13 @@ class LossContext:
         cur = torch.cuda.current_stream(phase.device)
         loss = torch.empty(1, dtype=torch.float64, device=phase.device)
         grad = torch.empty_like(phase) if want_grad else None
-        self.stream.wait_stream(cur)
+        other = cur != self.stream  # the same stream is ordered as it is
+        if other:
+            self.stream.wait_stream(cur)
         rc = B.gs_loss_grad_prepared(self.handle, phase.data_ptr(), loss.data_ptr(),
                                      grad.data_ptr() if grad is not None else 0)
-        cur.wait_stream(self.stream)
+        if other:
+            cur.wait_stream(self.stream)
         if rc != B.GS_OK:
             raise B.GSError(rc, "gs_loss_grad_prepared")
         return loss, grad
@@ -109,7 +115,7 @@ def _function():
         @staticmethod
         def backward(ctx, grad_out):
             (grad,) = ctx.saved_tensors
-            return grad * grad_out.to(grad.dtype), None, None
+            return grad * grad_out, None, None  # a scalar: the product has grad's type
 
     return IntensityLoss
 
