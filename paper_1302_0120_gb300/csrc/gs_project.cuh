@@ -14,6 +14,8 @@ namespace gsk {
 //   kProjTarget  z = Y:       z <- swap(m Y/|Y|)   (Eq. e:Mhat; a = m)
 //   kProjUnit    z = swap(v): z <- v/|v|           (Eq. e:PS with p = 1; a = 1)
 //   kProjSlm     z = swap(v): z <- p v/|v|         (Eq. e:PS; a = p)
+//   kProjSlmRg   the same in the register-resident general kernels, whose
+//                |z|^2 rounds the other product
 // with the phase of an exact zero taken as 0. amp[stride i] is the amplitude
 // at element i.
 //
@@ -21,7 +23,7 @@ namespace gsk {
 // root is the bare instruction and no zero rule applies: 9-10 instructions per
 // element. Otherwise the loop below it scales subnormals and selects zeros
 // (16 per element); both give the same bits on normal values.
-enum Projection { kProjTarget = 0, kProjUnit = 1, kProjSlm = 2 };
+enum Projection { kProjTarget = 0, kProjUnit = 1, kProjSlm = 2, kProjSlmRg = 3 };
 
 __device__ __forceinline__ float rsqrt_normal(float x) {
   float r;
@@ -29,10 +31,12 @@ __device__ __forceinline__ float rsqrt_normal(float x) {
   return r;
 }
 
-template <int PROJ, int V>
-__device__ __forceinline__ void project(float2 (&v)[V], float inv_sqrt_n, const float* amp, int stride, float& part) {
+// (v[0 .. V) of an array of M values)
+template <int PROJ, int V, int M>
+__device__ __forceinline__ void project(float2 (&v)[M], float inv_sqrt_n, const float* amp, int stride, float& part) {
+  static_assert(V <= M, "the values fit the array");
   auto sq = [](float2 z) {
-    return PROJ == kProjUnit ? norm2(z.y, z.x) : norm2(z.x, z.y);
+    return PROJ == kProjUnit || PROJ == kProjSlmRg ? norm2(z.y, z.x) : norm2(z.x, z.y);
   };
   bool normal = true;
 #pragma unroll

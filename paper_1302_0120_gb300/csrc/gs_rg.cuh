@@ -31,6 +31,7 @@
 
 #include "gs_common.cuh"
 #include "gs_general.cuh"
+#include "gs_project.cuh"
 #include "gs_rg_dft.cuh"
 #include "gs_tma.cuh"
 
@@ -184,8 +185,8 @@ __device__ __forceinline__ float run_pass_rg(const Params& p, int mb, int kind, 
     const float2* const twB = tw + NX;  // (V, T)
     for (int base = lo; base < hi; base += kThreads / 32) {
       const int idx = base + warp;
-      const bool valid = idx < hi;
-      const int ridx = valid ? idx : base;  // warps past the end work on a valid copy and store nothing
+      if (idx >= hi) break;  // warps past the end leave: a copy would only take issue slots
+      const int ridx = idx;
       const int tl = lane < T ? lane : 0;
       float2 v[M];
       if (kind == kInit) {
@@ -201,7 +202,7 @@ __device__ __forceinline__ float run_pass_rg(const Params& p, int mb, int kind, 
           const float a = pp ? pp[e] : 1.f;
           ex[e] = make_float2(a * c, a * s);
         }
-        if (last && valid) {  // zero iterations: the mask is arg exp(i phi^0)
+        if (last) {  // zero iterations: the mask is arg exp(i phi^0)
           float* po = p.phi_out + moff + static_cast<size_t>(idx) * NX;
 #pragma unroll 1
           for (int e = lane; e < NX; e += 32) po[e] = rg_phase(ex[e]);
@@ -219,20 +220,10 @@ __device__ __forceinline__ float run_pass_rg(const Params& p, int mb, int kind, 
       if (kind == kRow) {
         // v = swap(IDFT_x(B)) = swap(sqrt(N) P_M u^nu). Gap to S and Eq. (e:PS).
         const int ql = lane < V ? lane : 0;
-        const float* pp = p.p_slm ? p.p_slm + static_cast<size_t>(ridx) * NX + ql : nullptr;
-#pragma unroll
-        for (int j = 0; j < T; ++j) {
-          const float a = pp ? pp[V * j] : 1.f;
-          const float vx = v[j].y;
-          const float vy = v[j].x;
-          const float a2 = vx * vx + vy * vy;
-          const float rs = rsqrtf(a2);
-          const float mag = a2 > 0.f ? a2 * rs : 0.f;
-          const float d = mag * inv_sqrt_n - a;
-          part += d * d;
-          const float f = a * rs;
-          v[j] = a2 > 0.f ? make_float2(vx * f, vy * f) : make_float2(a, 0.f);
-        }
+        if (p.p_slm == nullptr)
+          project<kProjUnit, T>(v, inv_sqrt_n, nullptr, 0, part);
+        else
+          project<kProjSlmRg, T>(v, inv_sqrt_n, p.p_slm + static_cast<size_t>(ridx) * NX + ql, V, part);
         if (lane >= V) part = 0.f;
         if (last) {  // the mask, once per run, through the exchange buffer (element order)
           if (lane < V) {
@@ -240,7 +231,7 @@ __device__ __forceinline__ float run_pass_rg(const Params& p, int mb, int kind, 
             for (int j = 0; j < T; ++j) ex[lane + V * j] = v[j];
           }
           __syncwarp();
-          if (valid) {
+          {
             float* po = p.phi_out + moff + static_cast<size_t>(idx) * NX;
 #pragma unroll 1
             for (int e = lane; e < NX; e += 32) po[e] = rg_phase(ex[e]);
@@ -249,16 +240,16 @@ __device__ __forceinline__ float run_pass_rg(const Params& p, int mb, int kind, 
         }
         if (two) {
           rg_warp_dft<V, T>(v, ex, twB, lane);  // back to layout (T, V)
-          if (valid && lane < T) {
+          if (lane < T) {
 #pragma unroll
             for (int i = 0; i < V; ++i) Bm[L::off(idx, lane + T * i)] = v[i];
           }
         }
-      } else if (valid && lane < V) {  // kInit: B = DFT_x(u0), stored from layout (V, T)
+      } else if (lane < V) {  // kInit: B = DFT_x(u0), stored from layout (V, T)
 #pragma unroll
         for (int j = 0; j < T; ++j) Bm[L::off(idx, lane + V * j)] = v[j];
       }
-      if (valid) acc += part;
+      acc += part;
     }
     return acc;
   }
@@ -314,21 +305,8 @@ __device__ __forceinline__ float run_pass_rg(const Params& p, int mb, int kind, 
       const int ql = lane < V ? lane : 0;
       const float* mcol = ms + warp * NY + ql;
       float part = 0.f;
-#pragma unroll
-      for (int j = 0; j < T; ++j) {
-        const float m = mcol[V * j];
-        const float2 Y = v[j];
-        const float a2 = Y.x * Y.x + Y.y * Y.y;
-        const float rs = rsqrtf(a2);
-        const float mag = a2 > 0.f ? a2 * rs : 0.f;
-        const float d = mag * inv_sqrt_n - m;
-        part += d * d;
-        if (kind == kCol) {
-          const float f = m * rs;
-          const float2 Yh = a2 > 0.f ? make_float2(Y.x * f, Y.y * f) : make_float2(m, 0.f);
-          v[j] = make_float2(Yh.y, Yh.x);  // swapped: the next forward DFT acts as the inverse
-        }
-      }
+      // swapped: the next forward DFT acts as the inverse (kResid ends here)
+      project<kProjTarget, T>(v, inv_sqrt_n, mcol, V, part);
       if (lane < V) acc += part;
     }
     if (kind == kCol) {
