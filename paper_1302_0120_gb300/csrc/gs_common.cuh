@@ -135,6 +135,18 @@ static __device__ double block_sum_f(float x, Shared& sh) {
   return threadIdx.x == 0 ? block_total_f(sh) : 0.0;
 }
 
+// ... without holding up the block: the second warp adds the warps' totals and
+// writes *to, the others go on at once. Between two block barriers.
+static __device__ __forceinline__ void late_sum(float x, double* to, Shared& sh) {
+  warp_total_f(x, sh);
+  if (threadIdx.x >> 5 == 1) {
+    asm volatile("bar.sync 11, %0;" ::"r"(blockDim.x) : "memory");
+    if (threadIdx.x == 32) *to = block_total_f(sh);
+  } else {
+    asm volatile("bar.arrive 11, %0;" ::"r"(blockDim.x) : "memory");
+  }
+}
+
 // Sum of partials[row][0..G) in a fixed order (row = slot * batch + mask),
 // computed by one warp; the result is returned to every lane of that warp.
 static __device__ double warp_slot_sum(const Params& p, int row) {
@@ -166,15 +178,7 @@ static __device__ bool grid_sync(const Params& p, unsigned& target, Shared& sh, 
   }
   if (sum_to != nullptr) {  // the same in every thread
     __syncwarp();
-    warp_total_f(x, sh);
-    // the second warp adds the warps' totals; the others go on (thread 0 to
-    // the wait below)
-    if (threadIdx.x >> 5 == 1) {
-      asm volatile("bar.sync 11, %0;" ::"r"(blockDim.x) : "memory");
-      if (threadIdx.x == 32) *sum_to = block_total_f(sh);
-    } else {
-      asm volatile("bar.arrive 11, %0;" ::"r"(blockDim.x) : "memory");
-    }
+    late_sum(x, sum_to, sh);
   }
   if (threadIdx.x == 0) {
     int ok = 1;

@@ -35,7 +35,9 @@ constexpr float kTolDark = 3e-4f;  // t_d, Sec. II
 
 // partial-sum rows of the loss kernel (each [grid]); row kRowStaged holds the
 // reduced target statistics of a prepared target (flag, sum I, max I).
-enum LossRow { kRowFlag = 0, kRowSumI = 1, kRowMaxI = 2, kRowLoss = 3, kRowEl = 4, kRowEd = 5, kRowStaged = 6 };
+// The loss partials of the steps of a multi-step launch go alternately to the
+// two rows behind it (each of kMaxGrid).
+enum LossRow { kRowFlag = 0, kRowSumI = 1, kRowMaxI = 2, kRowLoss = 3, kRowEl = 4, kRowEd = 5, kRowStaged = 6, kRowSteps = 7 };
 
 // Record a failure: the first one also adds the abort bit to the barrier
 // counter, which releases every waiting block (as fail() in gs_common.cuh).
@@ -44,13 +46,23 @@ static __device__ void loss_fail(const LossParams& p, int code) {
   if (atomicExch(p.abort_flag, 1) == 0) atomicAdd(p.bar, kAbortBit);
 }
 
-// Grid barrier for the loss kernel (same protocol as grid_sync).
-static __device__ bool loss_sync(const LossParams& p, unsigned& target, Shared& sh) {
+// Grid barrier for the loss kernel (same protocol as grid_sync). With sum_to
+// the block's sum of x goes there behind the arrival, to be read after the
+// next barrier; `meanwhile` runs on the second warp's first thread while the
+// first warp waits.
+template <class F>
+static __device__ bool loss_sync(const LossParams& p, unsigned& target, Shared& sh, float x, double* sum_to,
+                                 F&& meanwhile) {
   __syncthreads();
   target += gridDim.x;
+  if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.bar) : "memory");
+  if (sum_to != nullptr) {  // the same in every thread
+    __syncwarp();
+    late_sum(x, sum_to, sh);
+  }
+  if (threadIdx.x == 32) meanwhile();
   if (threadIdx.x == 0) {
     int ok = 1;
-    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.bar) : "memory");
     unsigned spins = 0;
     unsigned long long t0 = 0;
     unsigned v;
@@ -72,6 +84,10 @@ static __device__ bool loss_sync(const LossParams& p, unsigned& target, Shared& 
   }
   __syncthreads();
   return sh.flag != 0;
+}
+
+static __device__ __forceinline__ bool loss_sync(const LossParams& p, unsigned& target, Shared& sh) {
+  return loss_sync(p, target, sh, 0.f, nullptr, [] {});
 }
 
 // The target's statistics from the blocks' partials, by one warp in a fixed
@@ -113,9 +129,11 @@ __global__ void __launch_bounds__(kThreads * kLossSplit, 1) gs_loss_kernel(const
   constexpr int W = L::W;
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Shared sh;
+  __shared__ float adam_c[2];  // Adam: lr / (1 - beta1^t), 1 / sqrt(1 - beta2^t)
   const int b = blockIdx.x;
   const int o = lane_of<kLossSplit>();  // this thread's lane of the block
   const int gidx = o >> LOGT;
+  const int team_line = (o & ~31) >> LOGT;  // the first line of this thread's team
   G grp;
   grp.t = o & (T - 1);
   grp.c = lane_part<kLossSplit>();
@@ -215,6 +233,7 @@ __global__ void __launch_bounds__(kThreads * kLossSplit, 1) gs_loss_kernel(const
     const int lo = split(b, gridDim.x, N);
     const int hi = split(b + 1, gridDim.x, N);
     for (int base = lo; base < hi; base += NG) {
+      if (base + team_line >= hi) break;  // no row for this team: a copy would only take issue slots
       const int idx = base + gidx;
       const bool valid = idx < hi;
       const int ridx = valid ? idx : base;
@@ -386,9 +405,13 @@ __global__ void __launch_bounds__(kThreads * kLossSplit, 1) gs_loss_kernel(const
       }
       if (want_grad && threadIdx.x == 0) bulk_wait_all();
     }
-    {
+    // FP32 within the block, FP64 across blocks (below). A step that another
+    // follows leaves its sum to the barrier, and block 0 adds the blocks' sums
+    // after the next one.
+    const bool fuse = k + 1 < steps;
+    double* const step_row = p.partials + (kRowSteps + (k & 1)) * kMaxGrid;
+    if (!fuse) {
       const int G = gridDim.x;
-      // FP32 within the block, FP64 across blocks (below)
       const double tot = block_sum_f(acc, sh);
       if (threadIdx.x == 0) p.partials[kRowLoss * G + b] = tot;
       if (want_phys) {
@@ -398,13 +421,20 @@ __global__ void __launch_bounds__(kThreads * kLossSplit, 1) gs_loss_kernel(const
         if (threadIdx.x == 0) p.partials[kRowEd * G + b] = td;
       }
     }
-    if (!loss_sync(p, target, sh)) {
+    if (!loss_sync(p, target, sh, acc, fuse ? step_row + b : nullptr, [&] {
+          if (!adam) return;
+          // the step's bias corrections, once per block (in every thread they
+          // took 0.5 us of a step)
+          const float t = static_cast<float>(t_done + 1 + k);
+          const float b1 = 1.f - powf(p.beta1, t);
+          const float b2 = 1.f - powf(p.beta2, t);
+          adam_c[0] = p.lr / b1;
+          adam_c[1] = 1.f / sqrtf(b2);
+        })) {
       if (threadIdx.x == 0 && sh.pending) mbar_wait_bounded(&sh.mbar, sh.pending_phase);
       return;
     }
-    // Block 0 reads the partials here and reaches the barrier that lets the
-    // other blocks write the next step's partials only after that.
-    if (b == 0 && threadIdx.x < 32) {
+    if (!fuse && b == 0 && threadIdx.x < 32) {
       const int G = gridDim.x;
       for (int row = kRowLoss; row <= (want_phys ? kRowEd : kRowLoss); ++row) {
         double s = 0.0;
@@ -427,21 +457,16 @@ __global__ void __launch_bounds__(kThreads * kLossSplit, 1) gs_loss_kernel(const
     // owns (the rows are split over the blocks as in pass 1): exp(i phi) of
     // the updated phase, straight from the update, then B = DFT_x through a
     // second turn of the transform loop.
-    const bool fuse = k + 1 < steps;
-    int adam_t = 0;
-    float adam_step = 0.f, adam_rb2 = 0.f;
-    if (adam) {
-      adam_t = t_done + 1 + k;
-      const float b1 = 1.f - powf(p.beta1, static_cast<float>(adam_t));
-      const float b2 = 1.f - powf(p.beta2, static_cast<float>(adam_t));
-      adam_step = p.lr / b1;
-      adam_rb2 = 1.f / sqrtf(b2);
-    }
+    const float adam_step = adam ? adam_c[0] : 0.f, adam_rb2 = adam ? adam_c[1] : 0.f;
     {
       const int lo = split(b, gridDim.x, N);
       const int hi = split(b + 1, gridDim.x, N);
       const float scale = 4.f * p.inv_n;
       for (int base = lo; base < hi; base += NG) {
+        // no row for this team (half of the teams at 512 x 512: 1.86 -> 1.68 ms
+        // per 100 steps; at 1024 x 1024 and above few are idle, and the loop
+        // that may end early was slower: 4.26 -> 4.57 ms per 200)
+        if (LN <= 9 && base + team_line >= hi) break;
         const int idx = base + gidx;
         const bool valid = idx < hi;
         const int ridx = valid ? idx : base;
@@ -535,7 +560,18 @@ __global__ void __launch_bounds__(kThreads * kLossSplit, 1) gs_loss_kernel(const
         grp.sync();
       }
     }
-    if (fuse && !loss_sync(p, target, sh)) return;
+    if (fuse) {
+      if (!loss_sync(p, target, sh)) return;
+      // block 0 reads the step's partials here; their row is written again two
+      // steps on, behind a barrier that block 0 reaches after this
+      if (b == 0 && threadIdx.x < 32) {
+        double s = 0.0;
+        for (int c = threadIdx.x; c < static_cast<int>(gridDim.x); c += 32) s += step_row[c];
+#pragma unroll
+        for (int o2 = 16; o2 > 0; o2 >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o2);
+        if (threadIdx.x == 0) p.loss[k] = s;
+      }
+    }
   }  // steps
   if (adam) {  // the last block to finish advances the step count (every block has read it)
     __syncthreads();
