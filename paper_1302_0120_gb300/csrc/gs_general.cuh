@@ -206,7 +206,8 @@ __device__ __forceinline__ void gen_build_amplitude(const Params& p, int mb, flo
     const int wc = min(8, hi - c0);
     if (k < wc)
       for (int y = threadIdx.x >> 3; y < ny; y += blockDim.x >> 3)
-        tile[k * (ny + 1) + y] = Im[static_cast<size_t>(y) * p.nx + c0 + k];
+        cp_async4(tile + k * (ny + 1) + y, Im + static_cast<size_t>(y) * p.nx + c0 + k);
+    cp_async_wait_all();
     __syncthreads();
     for (int c = 0; c < wc; ++c)
       for (int y = threadIdx.x; y < ny; y += blockDim.x)

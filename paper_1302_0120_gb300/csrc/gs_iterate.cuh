@@ -280,7 +280,7 @@ __device__ __forceinline__ float run_pass(const Params& p, int mb, int kind, boo
           for (int i = 0; i < V; ++i) cp_async4(&su[STEP * i].y, pp + STEP * i);
         }
         cp_async_wait_all();
-#pragma unroll 1
+#pragma unroll 4
         for (int i = 0; i < V; ++i) {
           float s, c;
           const float2 fa = su[STEP * i];
@@ -461,12 +461,15 @@ static __device__ void build_amplitude(const Params& p, int mb, float s, unsigne
   for (int base = lo; base < hi; base += W) {
     const int wcur = min(W, hi - base);
     __syncthreads();
+    // every copy of a thread in flight at once
     for (int e = threadIdx.x; e < p.ny * W; e += blockDim.x) {
       const int k = e & (W - 1);
       const int y = e >> logNG;
-      if (k < wcur) blk[y * (W + 1) + k] = Im[static_cast<size_t>(y) * p.nx + base + k];
+      if (k < wcur) cp_async4(blk + y * (W + 1) + k, Im + static_cast<size_t>(y) * p.nx + base + k);
     }
+    cp_async_wait_all();
     __syncthreads();
+#pragma unroll 4
     for (int e = threadIdx.x; e < wcur * p.ny; e += blockDim.x) {
       const int k = e >> p.logny;
       const int y = e & (p.ny - 1);
@@ -495,10 +498,17 @@ static __device__ __forceinline__ void a0_partials(const Params& p, Shared& sh) 
     const float* I = p.I + static_cast<size_t>(mb) * static_cast<size_t>(p.mstride) + static_cast<size_t>(r0) * p.nx;
     double acc = 0.0;
     bool bad = false;
-    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-      const float x = I[e];
-      bad |= !(x >= 0.f && x <= FLT_MAX);
-      acc += static_cast<double>(x);
+    constexpr int U = 8;  // loads in flight: one at a time, a 2048 x 2048 target took 50 us
+    const int step = blockDim.x;
+    for (int e0 = threadIdx.x; e0 < cnt; e0 += U * step) {
+      float x[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) x[u] = e0 + u * step < cnt ? I[e0 + u * step] : 0.f;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        bad |= !(x[u] >= 0.f && x[u] <= FLT_MAX);
+        acc += static_cast<double>(x[u]);
+      }
     }
     if (__syncthreads_or(bad)) acc = __longlong_as_double(0x7ff8000000000000ll);
     const double tot = block_sum(acc, sh);

@@ -68,11 +68,11 @@ __device__ __forceinline__ void project(float2 (&v)[M], float inv_sqrt_n, const 
   }
 }
 
-// The phases of a thread's values su[STEP i] in (-pi, pi]; a rolled loop
-// holds the only copy of atan2f.
+// The phases of a thread's values su[STEP i] in (-pi, pi]; the loop, four values
+// at a time, holds the only copies of atan2f.
 template <int V, int STEP>
 __device__ __forceinline__ void phase_out(float* po, const float2* su) {
-#pragma unroll 1
+#pragma unroll 4
   for (int i = 0; i < V; ++i) {
     const float2 u = su[STEP * i];
     const float ph = atan2f(u.y, u.x);

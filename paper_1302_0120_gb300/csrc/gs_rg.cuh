@@ -109,8 +109,9 @@ __device__ __forceinline__ void rg_build_amplitude(const Params& p, int mb, floa
     __syncthreads();
     for (int e = threadIdx.x; e < NY * W; e += kThreads) {
       const int y = e / W, k = e % W;
-      tile[y * (W + 1) + k] = Im[static_cast<size_t>(y) * NX + cb * W + k];
+      cp_async4(tile + y * (W + 1) + k, Im + static_cast<size_t>(y) * NX + cb * W + k);  // all in flight
     }
+    cp_async_wait_all();
     __syncthreads();
     for (int e = threadIdx.x; e < W * NY; e += kThreads) {
       const int k = e / NY, y = e % NY;

@@ -144,7 +144,7 @@ __device__ __forceinline__ float small_pass(const Params& p, size_t moff, int ki
   float2 v[V];
   if (kind == kSmallInit) {
     const float* ph = p.phi_in + moff + static_cast<size_t>(gline) * N + t0;
-#pragma unroll 1
+#pragma unroll 4
     for (int i = 0; i < V; ++i) {
       float s, c;
       sincosf(ph[STEP * i], &s, &c);
@@ -225,11 +225,17 @@ __global__ void __launch_bounds__(kSmallMaxThreads, 1) gs_small(const Params p) 
   // poisons it with NaN
   double acc = 0.0;
   bool bad = false;
-  const int share = Gm::N >> lc;
-  for (int e = threadIdx.x; e < share; e += nt) {
-    const float x = I[rank * share + e];
-    bad |= !(x >= 0.f && x <= FLT_MAX);
-    acc += static_cast<double>(x);
+  const int share = Gm::N >> lc;  // 32 values per lane, 8 per thread
+  constexpr int kPer = 32 / S;
+  {
+    float x[kPer];  // every load in flight
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) x[u] = I[rank * share + threadIdx.x + u * nt];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      bad |= !(x[u] >= 0.f && x[u] <= FLT_MAX);
+      acc += static_cast<double>(x[u]);
+    }
   }
   if (__syncthreads_or(bad)) acc = __longlong_as_double(0x7ff8000000000000ll);
 #pragma unroll
@@ -261,10 +267,16 @@ __global__ void __launch_bounds__(kSmallMaxThreads, 1) gs_small(const Params p) 
   {  // m of this block's columns
     float* const m = reinterpret_cast<float*>(smem + Gm::amp_at(lc));
     const int log_cols = LX - lc;
-    for (int e = threadIdx.x; e < share; e += nt) {
-      const int y = e >> log_cols;
-      const int x = e & ((1 << log_cols) - 1);
-      m[x * Gm::MLD + y] = s * sqrtf(I[y * Gm::NX + (rank << log_cols) + x]);
+    float v[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int e = threadIdx.x + u * nt;
+      v[u] = I[(e >> log_cols) * Gm::NX + (rank << log_cols) + (e & ((1 << log_cols) - 1))];
+    }
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+      const int e = threadIdx.x + u * nt;
+      m[(e & ((1 << log_cols) - 1)) * Gm::MLD + (e >> log_cols)] = s * sqrtf(v[u]);
     }
   }
   // stage twiddles of both lengths, held for the whole run
