@@ -850,9 +850,13 @@ int gs_physical_error(gs_ctx* c, const float* target_intensity, const float* pha
 int gs_set_slm_amplitude(gs_ctx* c, const float* amplitude) {
   if (c == nullptr || c->mixed) return GS_EINVAL;
   c->p_slm = amplitude;
+  // scratch: the last row of the partial sums, which no staged target and no
+  // run in progress on this stream holds
+  double* const scratch =
+      at<double>(c, c->L.partials) + (static_cast<size_t>(gsk::kSlots) * c->max_batch - 1) * gsk::kMaxGrid;
   if (amplitude != nullptr &&
-      gsk::launch_energy(amplitude, static_cast<long long>(c->nx) * c->ny, at<double>(c, c->L.energy), c->stream) !=
-          cudaSuccess) {
+      gsk::launch_energy(amplitude, static_cast<long long>(c->nx) * c->ny, at<double>(c, c->L.energy), scratch,
+                         c->stream) != cudaSuccess) {
     cudaGetLastError();
     c->p_slm = nullptr;
     return GS_ECUDA;

@@ -258,8 +258,9 @@ constexpr int kMaxAdamStepsPerLaunch = 1024;
 
 cudaError_t launch_loss(const LossParams& p, int grid, cudaStream_t s);
 cudaError_t launch_iterations(const Params& p, int grid, cudaStream_t s);
-// sum p^2 of an SLM amplitude into *energy (NaN if p has a negative or non-finite value)
-cudaError_t launch_energy(const float* p, long long n, double* energy, cudaStream_t s);
+// sum p^2 of an SLM amplitude into *energy (NaN if p has a negative or
+// non-finite value); scratch: kMaxGrid doubles
+cudaError_t launch_energy(const float* p, long long n, double* energy, double* scratch, cudaStream_t s);
 cudaError_t iteration_occupancy(int nx, int ny, int* blocks_per_sm, int tc_mode = kTcNone);
 // The tcgen05 kernel of n x n masks, log2(n) = l in 8..10 (gs_tc5_inst.cu);
 // FP16 or BF16 operands; null for other sizes.
