@@ -1,0 +1,93 @@
+"""The ways a pass can be organised: clusters of one to eight blocks for small
+grids, one or two threads per lane, one to four column blocks in flight, rounds
+whose copies start during the round before. Every one evaluates the same
+butterflies and projections, so the phases of a run agree bit for bit whichever
+way its grid, batch and block count select; the gaps agree to the rounding of
+the block sums. The short form of the projections (all values normal) and the
+long one (zeros) are compared with the oracle."""
+
+import numpy as np
+import pytest
+
+import oracle.gs_oracle as O
+from paper_1302_0120_gb300 import synthetic as S
+from tests.gpu_util import GROUPING_RTOL, aligned_rel_err, gpu_gs
+from tests.test_gpu_batch import make_batch, run_batched
+
+pytestmark = pytest.mark.gpu
+
+
+def _same(a, b):
+    assert a[3] == 0 and b[3] == 0
+    assert np.array_equal(a[0], b[0]), np.max(np.abs(a[0] - b[0]))
+    np.testing.assert_allclose(a[1], b[1], rtol=GROUPING_RTOL, atol=0)
+    np.testing.assert_allclose(a[2], b[2], rtol=GROUPING_RTOL, atol=0)
+
+
+# masks of a batch: the cluster shrinks as the batch grows (64 x 64: four blocks
+# for one mask, two for 64; 128 x 128: eight, four, then the persistent kernel)
+@pytest.mark.parametrize("ny,nx,masks", [
+    (32, 32, 1), (32, 32, 64), (64, 64, 64), (256, 32, 20), (64, 256, 2), (128, 128, 1), (128, 128, 30),
+    (128, 128, 60), (128, 256, 1), (256, 128, 12), (256, 128, 40),
+])
+def test_clusters_match_persistent_kernel(ny, nx, masks):
+    I, P = make_batch(masks, ny, nx, nspots=4)
+    got = run_batched(I, P, 5)
+    ref = run_batched(I, P, 5, grid=5)
+    _same(got, ref)
+
+
+# few blocks make every pass several rounds, the last one ragged; None is the
+# grid that a run chooses (one round for these masks)
+@pytest.mark.parametrize("ny,nx,grid", [
+    (1024, 1024, 9), (1024, 1024, 41), (512, 512, 7), (256, 256, 3), (512, 1024, 11), (1024, 256, 6),
+    (2048, 1024, 23), (64, 2048, 3), (128, 512, 1),
+])
+def test_rounds_match_one_round(ny, nx, grid):
+    I = S.spot_target(41, ny, nx, 9, (0.5, 1.0))
+    phi0 = S.random_phase(42, ny, nx)
+    _same(gpu_gs(I, phi0, 4), gpu_gs(I, phi0, 4, grid=grid))
+
+
+# batches of one grid and of single runs, on the grid of the whole batch
+@pytest.mark.parametrize("masks,ny,nx", [(9, 1024, 1024), (11, 512, 512), (17, 256, 256), (3, 2048, 1024),
+                                         (5, 600, 800), (4, 250, 360), (3, 1024, 1280)])
+def test_batches_match_single_runs(masks, ny, nx):
+    I, P = make_batch(masks, ny, nx, nspots=8)
+    ph, r, g, st = run_batched(I, P, 3)
+    for k in (0, masks // 2, masks - 1):
+        _same((ph[k], r[k], g[k], st), gpu_gs(I[k], P[k], 3))
+
+
+# A constant start transforms to a single frequency: the other values of F u are
+# exact zeros on these grids, which take phase 0 (zero rule of the projections).
+@pytest.mark.parametrize("n,grid", [(64, None), (64, 2), (128, None), (256, None), (512, None), (1024, None)])
+def test_exact_zeros_take_phase_zero(n, grid):
+    I = S.spot_target(51, n, n, 7, (0.5, 1.0))
+    phi0 = np.zeros((n, n), np.float32)
+    ph, r, g, st = gpu_gs(I, phi0, 1, grid=grid)
+    assert st == 0
+    # the oracle's transform leaves residues of 1e-16 where the exact one has
+    # zeros: the step from the exact spectrum instead, F u0 = N at DC only
+    m = O.target_amplitude(I)
+    v = np.fft.ifft2(m) * n
+    # v is real, so that the phase of its smallest values is all rounding: with
+    # an FP32 error of 5e-7 rms in v, the pixels above 0.05 rms are off by 2e-6
+    # in the root mean square (E[1/v^2] = 16 there)
+    keep = np.abs(v) > 0.05 * np.sqrt(np.mean(np.abs(v) ** 2))
+    assert aligned_rel_err(ph[keep], (v / np.abs(v))[keep]) <= 1e-5
+    r0 = np.sqrt(((np.where(np.arange(n * n).reshape(n, n) == 0, float(n), 0.0) - m) ** 2).sum()) / n
+    assert abs(r[0] - r0) <= 1e-5 * r0
+
+
+@pytest.mark.parametrize("ny,nx", [(1024, 1280), (480, 640), (1500, 1500), (9, 1536)])
+def test_general_teams_parity(ny, nx):
+    I = S.spot_target(61, ny, nx, 6, (0.5, 1.0)) if min(ny, nx) > 20 else np.eye(ny, nx, 5, dtype=np.float32)
+    phi0 = S.random_phase(62, ny, nx)
+    ph, r, g, st = gpu_gs(I, phi0, 2)
+    assert st == 0
+    ref = O.gs_run(I, phi0, 2)
+    np.testing.assert_allclose(r, ref["r"], rtol=1e-3)
+    one = gpu_gs(I, phi0, 1)[0]
+    u, _, _ = O.gs_step(np.exp(1j * phi0.astype(np.float64)), O.target_amplitude(I))
+    assert aligned_rel_err(one, u) <= 1e-5
