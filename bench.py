@@ -677,7 +677,7 @@ def run_gpu(args):
                 host6.append(1e3 * (time.perf_counter() - t0))
         if g6.status() != 0 or g6p.status() != 0 or g6b.status() != 0:
             raise RuntimeError("64x64 runs failed")
-        spots64 = {"iters": K6, "kernel": "one block per mask, field in shared memory",
+        spots64 = {"iters": K6, "kernel": "one cluster per mask, field in shared memory",
                    "device_ms": round(ms_small, 4), "e2e_ms": round(statistics.mean(host6), 4),
                    "persistent_kernel_ms": round(ms_pers, 4), "persistent_grid_ctas": g6p.grid,
                    "batch64_ms": round(ms_batch, 4), "batch64_masks_per_s": round(64e3 / ms_batch, 1),
