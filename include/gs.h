@@ -354,7 +354,9 @@ int gs_set_grid(gs_ctx* c, int ctas);
 int gs_test_barrier_timeout(gs_ctx* c, int enable);
 
 /*
- * gs_get_grid -- the number of thread blocks the next run will launch.
+ * gs_get_grid -- the number of thread blocks of the persistent kernel for a
+ * run of one mask. A batch may take more of them, and a run on the small-grid
+ * kernel (see gs_run) takes its clusters instead.
  * Writes it to *ctas (host). Returns GS_EINVAL for NULL arguments.
  */
 int gs_get_grid(gs_ctx* c, int* ctas);

@@ -286,8 +286,7 @@ int check_guards(const unsigned char* ws, const Layout& L) {
 // log2 of the blocks per mask of a small-grid run: the most for which every
 // block of the batch has an SM (64 masks of 64 x 64 x 20 iterations: 110 us
 // with two blocks each, 125 with four that share SMs). Without any, the fewest
-// blocks,
-// where shared memory has room for the grid on one or two SMs (at most 8192
+// blocks, where shared memory has room for the grid on one or two SMs (at most 8192
 // pixels); larger grids then run on the persistent kernel (-1), which shares
 // the device between the masks.
 int small_logc(const gs_ctx* c, int batch) {
