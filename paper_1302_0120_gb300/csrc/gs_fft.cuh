@@ -24,9 +24,10 @@ __host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return mak
 // a * w for a twiddle w = (c, s) meaning c + i s. The fused operations are
 // written out here and in norm2: left to the compiler, the choice of the
 // product that is fused depends on the code around it, and the same
-// transform would round differently from kernel to kernel. (cmul_late: the
-// stage after 1024 points, which fuses the other product of the imaginary
-// part.)
+// transform would round differently from kernel to kernel. (cmul_late fuses
+// the other product of the imaginary part: the stage after 1024 points, and
+// the twiddles of both tensor-core transforms, which then give the same masks
+// bit for bit.)
 __host__ __device__ __forceinline__ float2 cmul(float2 a, float2 w) {
   return make_float2(fmaf(a.x, w.x, -(a.y * w.y)), fmaf(a.y, w.x, a.x * w.y));
 }

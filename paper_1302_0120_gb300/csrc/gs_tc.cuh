@@ -246,8 +246,8 @@ struct TcFft {
           const int slot = ((mp * 4 + nt) * 2 + h) * 2;
           const float2 w0 = tw[slot * 32 + lane];
           const float2 w1 = tw[(slot + 1) * 32 + lane];
-          const float2 y0 = cmul(make_float2(acc[mp][nt][2 * h], acc[mp + 2][nt][2 * h]), w0);
-          const float2 y1 = cmul(make_float2(acc[mp][nt][2 * h + 1], acc[mp + 2][nt][2 * h + 1]), w1);
+          const float2 y0 = cmul_late(make_float2(acc[mp][nt][2 * h], acc[mp + 2][nt][2 * h]), w0);
+          const float2 y1 = cmul_late(make_float2(acc[mp][nt][2 * h + 1], acc[mp + 2][nt][2 * h + 1]), w1);
           z[0][nt][mp][h] = pack_h2(y0.x, y1.x);
           z[1][nt][mp][h] = pack_h2(y0.y, y1.y);
         }

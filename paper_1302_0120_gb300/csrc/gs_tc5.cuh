@@ -353,9 +353,9 @@ struct Tc5Fft {
       for (int j = 0; j < 8; ++j) {
         const int k1 = 8 * g + j;
         const float2 w = twl[32 * k1];
-        const float a = d[k1], b = d[32 + k1];
-        zr[j] = a * w.x - b * w.y;
-        zi[j] = a * w.y + b * w.x;
+        const float2 z = cmul_late(make_float2(d[k1], d[32 + k1]), w);  // rounds as the mma.sync form
+        zr[j] = z.x;
+        zi[j] = z.y;
       }
       const int c = (8 * g) / R;
       const int m = 32 * wq + R * gam + (8 * g) % R;

@@ -187,3 +187,18 @@ def test_large_laser_amplitude_is_rescaled(n, engine):
     u_ref, _, _ = O.gs_step(100.0 * np.exp(1j * start.astype(np.float64)), O.target_amplitude(I, energy=float(n * n) * 1e4),
                             p.astype(np.float64))
     assert aligned_rel_err(nxt, u_ref / 100.0) <= STEP_TOL
+
+
+@pytest.mark.parametrize("n,laser", [(256, False), (512, False), (1024, False), (512, True)])
+def test_fp16_engines_give_the_same_masks(n, laser):
+    """tcgen05 and mma.sync with FP16 operands round the same operands (inputs,
+    twiddled stage-1 products) and accumulate in FP32: the masks of a run are
+    equal bit for bit, and the gaps to the rounding of the block sums."""
+    I, phi0 = S.spot_target(120 + n, n, n, 30, (0.5, 1.0)), S.random_phase(121 + n, n, n)
+    p = S.laser_amplitude(n, n) if laser else None
+    a = tc_run(I, phi0, 10, p=p)
+    b = tc_run(I, phi0, 10, p=p, engine="mma-sync")
+    assert a[3] == 0 and b[3] == 0
+    assert np.array_equal(a[0], b[0]), int((a[0] != b[0]).sum())
+    for x, y in zip(a[1:3], b[1:3]):
+        np.testing.assert_allclose(x, y, rtol=GROUPING_RTOL, atol=0)
