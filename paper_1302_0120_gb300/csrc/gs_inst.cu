@@ -25,4 +25,15 @@ const void* iterate_kernel_lx<GS_LX>(int ly) {
   }
 }
 
+#if GS_LX >= 11
+template <>
+const void* iterate_kernel_slm_lx<GS_LX>(int ly) {
+  if (ly == 12) return reinterpret_cast<const void*>(gs_iterate<GS_LX, 12, false, true>);
+#if GS_LX == 12
+  if (ly == 11) return reinterpret_cast<const void*>(gs_iterate<GS_LX, 11, false, true>);
+#endif
+  return nullptr;
+}
+#endif
+
 }  // namespace gsk

@@ -186,6 +186,10 @@ inline GenGeom gen_geom(int nx, int ny, int masks, int sms) {
 // Kernel for log2(nx) = LX and the given log2(ny); defined per LX in gs_inst.cu.
 template <int LX>
 const void* iterate_kernel_lx(int ly);
+// Kernel of runs under a laser amplitude for log2(nx) = LX in 11, 12; null where
+// the kernel above serves them.
+template <int LX>
+const void* iterate_kernel_slm_lx(int ly);
 // Kernel with tensor-core transforms for an n x n grid, log2(n) = l in 8..10
 // (gs_tc_inst.cu); null otherwise.
 const void* iterate_kernel_tc(int l);

@@ -55,11 +55,14 @@ constexpr int kTcCsOffset = kTcTwOffset + kTcTwBytes;
 static_assert(kTcTwBytes + kTcCsBytes == kTcExtraSmemBytes, "tensor-core tables match the launch size");
 
 // Stands in for TcFft in the kernels whose transforms run on the FP32 ALUs,
-// S threads per lane; AHEAD: the kernel has the second staging buffer.
-template <int S, bool AHEAD = S == 1>
+// S threads per lane; AHEAD: the kernel has the second staging buffer; SLM: the
+// kernel of runs under a laser amplitude (iterate_kernel_slm).
+template <int S, bool AHEAD = S == 1, bool SLM = false>
 struct NoTc {
+  static_assert(!SLM || AHEAD, "the laser amplitude takes the second staging buffer");
   static constexpr int kThreadsPerLane = S;
   static constexpr bool kAhead = AHEAD;
+  static constexpr bool kSlm = SLM;
   static constexpr bool kEnabled = false;
   static constexpr bool kTcgen05 = false;
 };
@@ -69,6 +72,12 @@ template <class TCF>
 __host__ __device__ constexpr bool loads_ahead() {
   if constexpr (TCF::kEnabled) return false;
   else return TCF::kAhead;
+}
+
+template <class TCF>
+__host__ __device__ constexpr bool slm_kernel() {
+  if constexpr (TCF::kEnabled) return false;
+  else return TCF::kSlm;
 }
 
 // Threads per lane of a kernel whose transforms are TCF's.
@@ -245,11 +254,13 @@ __device__ __forceinline__ float run_pass(const Params& p, int mb, int kind, boo
   // Row passes of several rounds fetch the next round's rows (16-byte pieces)
   // into the field staging buffer behind the transforms of this round; a
   // group's row sits at its own N elements of the buffer.
-  const bool fetch = !TCF::kEnabled && L::W >= 2 && kind == kRow && p.p_slm == nullptr;
+  constexpr bool kSlm = slm_kernel<TCF>();
+  const bool fetch = !TCF::kEnabled && L::W >= 2 && kind == kRow && (kSlm || p.p_slm == nullptr);
   float2* const next_row = blk + g * N;
   // the laser amplitude of a row, at this thread's elements (in the field
-  // staging buffer, free in row passes)
-  float* const sp = reinterpret_cast<float*>(blk) + threadIdx.x;
+  // staging buffer, free in row passes; in the second one where the first
+  // holds the next rows)
+  float* const sp = reinterpret_cast<float*>(kSlm ? blk + kBlockElems : blk) + threadIdx.x;
 
   for (int u0 = lo; u0 < hi; u0 += rows ? NG : P) {
     const int idx = rows ? u0 + g : u0 + slot;  // this group's row, or this slot's column block
@@ -777,8 +788,8 @@ __host__ __device__ constexpr int kernel_split() {
   return (TC || LX == 0) ? 1 : iteration_split(1 << LX, 1 << LY);
 }
 
-// One size class per launch (every grid).
-template <int LX, int LY, bool TC = false>
+// One size class per launch (every grid). SLM: iterate_kernel_slm.
+template <int LX, int LY, bool TC = false, bool SLM = false>
 __global__ void __launch_bounds__(LX == 0 ? kGenMaxThreads : kThreads * kernel_split<LX, LY, TC>(), 1) gs_iterate(const Params p) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ Shared sh;
@@ -804,7 +815,7 @@ __global__ void __launch_bounds__(LX == 0 ? kGenMaxThreads : kThreads * kernel_s
   }
   const auto tcf = [&]() {
     if constexpr (TC) return TcFft<LX>{s1, s2, tctw};
-    else return NoTc<S>{};
+    else return NoTc<S, S == 1, SLM>{};
   }();
   iterate_class<LX, LY, kHold>(p, sh, smem, tw_rows, tcf);
 }

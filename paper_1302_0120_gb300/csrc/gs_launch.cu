@@ -64,6 +64,8 @@ extern template const void* iterate_kernel_lx<9>(int);
 extern template const void* iterate_kernel_lx<10>(int);
 extern template const void* iterate_kernel_lx<11>(int);
 extern template const void* iterate_kernel_lx<12>(int);
+extern template const void* iterate_kernel_slm_lx<11>(int);
+extern template const void* iterate_kernel_slm_lx<12>(int);
 
 extern template const void* iterate_kernel_rg_nx<600>(int);
 extern template const void* iterate_kernel_rg_nx<768>(int);
@@ -122,6 +124,21 @@ static const void* kernel_for(int nx, int ny, int tc_mode) {
   }
 }
 
+// Runs under a laser amplitude whose row passes take seven rounds or more
+// (256 / (nx/32) rows per block and round: 4096 x 4096, 4096 x 2048 and 2048 x
+// 4096) have a kernel of their own, which fetches the next rows behind the
+// transforms as the kernel of p = 1 does and keeps the row's amplitude in the
+// second staging buffer. nx x ny x 10 iterations without and with the fetch:
+// 4096 x 4096 3.78 and 3.20 ms, 4096 x 2048 1.36 and 1.30, 2048 x 4096 1.72 and
+// 1.47; with four rounds it is slower (2048 x 2048 0.696 and 0.700, 4096 x 1024
+// 0.632 and 0.639). One kernel that chooses at run time cost p = 1 one per cent
+// (4096 x 4096 3.01 and 3.04). Null: the common kernel.
+static const void* iterate_kernel_slm(int nx, int ny, int tc_mode) {
+  if (tc_mode != kTcNone || uses_general(nx, ny)) return nullptr;
+  if (nx == 4096) return iterate_kernel_slm_lx<12>(log2_exact(ny));
+  return nx == 2048 ? iterate_kernel_slm_lx<11>(log2_exact(ny)) : nullptr;
+}
+
 // threads per block of the kernel of an nx x ny grid (not the general kernel,
 // whose block depends on the run)
 static int iteration_threads(int nx, int ny, int tc_mode) {
@@ -151,6 +168,10 @@ cudaError_t iteration_occupancy(int nx, int ny, int* blocks_per_sm, int tc_mode)
   const size_t allow = (uses_general(nx, ny) && !uses_rg(nx, ny)) ? kGenSmemLimit : smem;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(allow));
   if (e != cudaSuccess) return e;
+  if (const void* ks = iterate_kernel_slm(nx, ny, tc_mode)) {  // the same shared memory: one block per SM, as k
+    e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e != cudaSuccess) return e;
+  }
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, iteration_threads(nx, ny, tc_mode), smem);
 }
 
@@ -178,7 +199,8 @@ cudaError_t launch_mixed(const MixedParams& mp, int grid, int tc_mode, cudaStrea
 }
 
 cudaError_t launch_iterations(const Params& p, int grid, cudaStream_t s) {
-  const void* k = kernel_for(p.nx, p.ny, p.tensor_core);
+  const void* k = p.p_slm != nullptr ? iterate_kernel_slm(p.nx, p.ny, p.tensor_core) : nullptr;
+  if (k == nullptr) k = kernel_for(p.nx, p.ny, p.tensor_core);
   if (k == nullptr) return cudaErrorInvalidValue;
   void* args[] = {const_cast<Params*>(&p)};
   if (p.gen_teams > 0)

@@ -91,3 +91,77 @@ def test_general_teams_parity(ny, nx):
     one = gpu_gs(I, phi0, 1)[0]
     u, _, _ = O.gs_step(np.exp(1j * phi0.astype(np.float64)), O.target_amplitude(I))
     assert aligned_rel_err(one, u) <= 1e-5
+
+
+def _laser_with_dark_pixels(ny, nx):
+    """A beam profile with some pixels switched off (p = 0)."""
+    p = S.laser_amplitude(ny, nx)
+    p[::7, ::5] = 0.0
+    return p
+
+
+def _laser_run(I, P, p, iters, grid=None, masks=1):
+    import torch
+
+    from paper_1302_0120_gb300 import GerchbergSaxton, build_lib
+    from paper_1302_0120_gb300 import _binding as B
+
+    build_lib.build()
+    ny, nx = I.shape[-2:]
+    It, Pt, pt = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (I, P, p))
+    with GerchbergSaxton(nx, ny, max_batch=masks) as gs:
+        gs.set_slm_amplitude(pt)
+        if grid:
+            gs.set_grid(grid)
+        out = gs.run(It, Pt, iters) if masks == 1 else gs.run_batched(It, Pt, iters)
+        st = gs.status()
+        assert B.gs_check_workspace(gs.handle) == B.GS_OK
+        return tuple(x.cpu().numpy() for x in out) + (st,)
+
+
+# Under a laser amplitude a row pass stages the row's amplitude in shared memory
+# beside the fetched rows or in their place: rounds after the first, for two
+# threads a lane, one, and the grids with a kernel of their own (nx = 4096 and
+# ny >= 2048, 2048 x 4096; several rounds on any grid).
+@pytest.mark.parametrize("ny,nx,grid", [(64, 64, 1), (512, 512, 7), (1024, 1024, 9), (2048, 1024, 23), (600, 800, 11),
+                                        (2048, 4096, 37), (4096, 2048, 41)])
+def test_laser_rounds_match_one_round(ny, nx, grid):
+    I = S.spot_target(71, ny, nx, 9, (0.5, 1.0))
+    phi0 = S.random_phase(72, ny, nx)
+    p = _laser_with_dark_pixels(ny, nx)
+    _same(_laser_run(I, phi0, p, 3), _laser_run(I, phi0, p, 3, grid=grid))
+
+
+@pytest.mark.parametrize("masks,ny,nx", [(9, 1024, 1024), (11, 512, 512), (3, 600, 800)])
+def test_laser_batches_match_single_runs(masks, ny, nx):
+    I, P = make_batch(masks, ny, nx, nspots=8)
+    p = _laser_with_dark_pixels(ny, nx)
+    ph, r, g, st = _laser_run(I, P, p, 3, masks=masks)
+    for k in (0, masks // 2, masks - 1):
+        _same((ph[k], r[k], g[k], st), _laser_run(I[k], P[k], p, 3))
+
+
+# One step in FP64 (torch.fft) on the grids whose laser runs have a kernel of
+# their own, and their neighbours on the common one. The FP32 step's error there
+# is some 1e-6 in the root mean square (as for p = 1, test_gpu_parity.py).
+@pytest.mark.parametrize("ny,nx", [(4096, 4096), (2048, 4096), (4096, 2048), (1024, 4096), (2048, 2048)])
+def test_laser_step_on_long_rows(ny, nx):
+    import torch
+
+    I = S.spot_target(73, ny, nx, 20, (0.5, 1.0))
+    phi0 = S.random_phase(74, ny, nx)
+    p = _laser_with_dark_pixels(ny, nx)
+    ph, r, g, st = _laser_run(I, phi0, p, 1)
+    assert st == 0
+    I64, phi64, p64 = (torch.from_numpy(x).cuda().double() for x in (I, phi0, p))
+    energy = (p64 * p64).sum()
+    m = torch.sqrt(I64 * (energy / I64.sum()))
+    Y = torch.fft.fft2(torch.polar(p64, phi64)) / (ny * nx) ** 0.5
+    v = torch.fft.ifft2(torch.polar(m, torch.angle(Y))) * (ny * nx) ** 0.5
+    r0 = float(torch.sqrt(((Y.abs() - m) ** 2).sum() / energy))
+    g0 = float(torch.sqrt(((v.abs() - p64) ** 2).sum() / energy))
+    assert abs(r[0] - r0) <= 1e-5 * r0 and abs(g[0] - g0) <= 1e-5 * g0
+    a = torch.polar(p64, torch.from_numpy(ph).cuda().double())
+    b = torch.polar(p64, torch.angle(v))
+    c = (a.conj() * b).sum()
+    assert float(torch.linalg.norm(a * (c / c.abs()) - b) / torch.linalg.norm(b)) <= 1e-5
