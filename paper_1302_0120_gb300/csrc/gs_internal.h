@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <initializer_list>
+
 namespace gsk {
 
 // A block of the iteration kernels works on 256 lanes of 32 values, each held
@@ -144,6 +146,7 @@ constexpr int kMaxGeneralStages = 10;
 
 // The general kernel transforms a row or column with a team of threads; a
 // block has at most kGenMaxTeams teams, and one block runs per SM.
+constexpr int kGenMinTeams = 4;
 constexpr int kGenMaxTeams = 10;
 constexpr int kGenMaxThreads = 640;
 static_assert(kGenMaxTeams << 6 <= kGenMaxThreads, "teams of two warps fit");
@@ -159,10 +162,23 @@ inline __host__ __device__ size_t gen_smem_bytes(int nx, int ny, int teams) {
          sizeof(float2);
 }
 
+// Values that the busiest thread of a team of `threads` threads takes through
+// shared memory in a length-n transform: R per butterfly and stage (the radices
+// of radix_plan, gs_api.cu).
+inline int gen_thread_values(int n, int threads) {
+  int left = n, sum = 0;
+  for (int r : {3, 5, 8, 4, 2})
+    while (left % r == 0) {
+      sum += r * ((n / r + threads - 1) / threads);
+      left /= r;
+    }
+  return sum;
+}
+
 // Teams per block and log2 of a team's threads for `masks` masks of nx x ny
 // on `sms` SMs: the fewest rounds that shared memory allows, then the fewest
-// teams that need no more (at least 4, so that column tiles are 32-byte row
-// segments).
+// teams that need no more (at least kGenMinTeams, so that column tiles are
+// 32-byte row segments).
 struct GenGeom {
   int teams;
   int team_log;
@@ -170,16 +186,24 @@ struct GenGeom {
 inline GenGeom gen_geom(int nx, int ny, int masks, int sms) {
   const int nmax = nx > ny ? nx : ny;
   int fit = kGenMaxTeams;
-  while (fit > 4 && gen_smem_bytes(nx, ny, fit) > static_cast<size_t>(kGenSmemLimit)) --fit;
+  while (fit > kGenMinTeams && gen_smem_bytes(nx, ny, fit) > static_cast<size_t>(kGenSmemLimit)) --fit;
   const long long lines = static_cast<long long>(nmax) * masks;
   const long long rounds = (lines + static_cast<long long>(sms) * fit - 1) / (static_cast<long long>(sms) * fit);
   const long long per = static_cast<long long>(sms) * rounds;
   int teams = static_cast<int>((lines + per - 1) / per);
-  if (teams < 4) teams = 4;
-  // two warps per line; four for the longer ones, where a block has room
-  // (640 x 480: 384 -> 374 us per 20 iterations; 120 x 90: 246 -> 272)
-  int tl = nmax >= 300 ? 7 : 6;
-  if ((teams << tl) > kGenMaxThreads) tl = 6;
+  if (teams < kGenMinTeams) teams = kGenMinTeams;
+  // Two warps per line. Four, where a block has room, if they spare the
+  // busiest thread of a row and of a column transform 23 values together: that
+  // pays for the wider synchronisation of every stage. Ten iterations with two
+  // warps and four, values spared: 320 x 320 (0) 147 and 164 us, 384 x 384 (10)
+  // 167 and 179, 480 x 320 (12) 161 and 168, 400 x 300 (21) 168 and 170, 480 x
+  // 360 (23) 173 and 172, 600 x 50 (24) 154 and 150, 400 x 400 (28) 180 and
+  // 182, 432 x 324 (29) 186 and 182, 500 x 375 (37) 177 and 170, 640 x 480 (37)
+  // 204 and 200, 625 x 625 (40) 220 and 207. Sides below 300 keep two (243 x
+  // 243, 30 spared: 170 and 171).
+  const int saved = gen_thread_values(nx, 64) + gen_thread_values(ny, 64) - gen_thread_values(nx, 128) -
+                    gen_thread_values(ny, 128);
+  const int tl = nmax >= 300 && saved >= 23 && (teams << 7) <= kGenMaxThreads ? 7 : 6;
   return {teams, tl};
 }
 
