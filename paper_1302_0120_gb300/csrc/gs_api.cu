@@ -298,18 +298,33 @@ int small_logc(const gs_ctx* c, int batch) {
 
 bool on_general(const gs_ctx* c) { return !c->mixed && gsk::uses_general(c->nx, c->ny) && !gsk::uses_rg(c->nx, c->ny); }
 
+// Blocks of a run on the general kernel, and their geometry.
+struct GenRun {
+  gsk::GenGeom geom;
+  int grid;
+};
+GenRun gen_run(const gs_ctx* c, int masks) {
+  GenRun r{gsk::gen_geom(c->nx, c->ny, masks, c->num_sms), 0};
+  if (c->grid_override > 0) {
+    // A fixed grid may put several blocks on an SM (max_grid): smaller ones
+    // then, those whose occupancy the context has asked for.
+    const int cap = max_grid(c);
+    r.grid = c->grid_override < cap ? c->grid_override : cap;
+    if (r.grid > c->num_sms) r.geom = gsk::kGenMinGeom;
+    return r;
+  }
+  // one block per SM at most, enough for one line per team and round
+  const long long lines = static_cast<long long>(c->nx > c->ny ? c->nx : c->ny) * masks;
+  const long long g = (lines + r.geom.teams - 1) / r.geom.teams;
+  r.grid = static_cast<int>(g < c->num_sms ? g : c->num_sms);
+  return r;
+}
+
 // Blocks of a run of `masks` masks iterated together: a pass splits the rows
 // or column blocks of all of them over the grid, so the rule counts their
 // pixels (4 masks of 512 x 512 on 64 blocks: 28 us per iteration, on 152: 15).
 int choose_grid(const gs_ctx* c, int masks) {
-  if (on_general(c)) {
-    // one block per SM at most, enough for one line per team and round
-    if (c->grid_override > 0) return c->grid_override < c->num_sms ? c->grid_override : c->num_sms;
-    const gsk::GenGeom gg = gsk::gen_geom(c->nx, c->ny, masks, c->num_sms);
-    const long long lines = static_cast<long long>(c->nx > c->ny ? c->nx : c->ny) * masks;
-    const long long g = (lines + gg.teams - 1) / gg.teams;
-    return static_cast<int>(g < c->num_sms ? g : c->num_sms);
-  }
+  if (on_general(c)) return gen_run(c, masks).grid;
   return choose_grid_for(c, static_cast<long long>(c->nx) * c->ny * masks);
 }
 
@@ -438,7 +453,7 @@ int gs_run_batched(gs_ctx* c, int batch, const float* target_intensity, const fl
   radix_plan(c->nx, &p.planx, &p.nstx);
   radix_plan(c->ny, &p.plany, &p.nsty);
   if (on_general(c)) {
-    const gsk::GenGeom gg = gsk::gen_geom(c->nx, c->ny, group, c->num_sms);
+    const gsk::GenGeom gg = gen_run(c, group).geom;
     p.gen_teams = gg.teams;
     p.gen_team_log = gg.team_log;
   }

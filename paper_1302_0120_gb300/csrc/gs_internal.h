@@ -183,6 +183,10 @@ struct GenGeom {
   int teams;
   int team_log;
 };
+// The smallest block, the one of which an SM may hold several: kThreads
+// threads (iteration_threads) and gen_smem_bytes(nx, ny, kGenMinTeams).
+constexpr GenGeom kGenMinGeom{kGenMinTeams, 6};
+static_assert(kGenMinGeom.teams << kGenMinGeom.team_log == kThreads, "the block of the occupancy query");
 inline GenGeom gen_geom(int nx, int ny, int masks, int sms) {
   const int nmax = nx > ny ? nx : ny;
   int fit = kGenMaxTeams;

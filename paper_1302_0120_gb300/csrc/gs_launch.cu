@@ -139,8 +139,8 @@ static const void* iterate_kernel_slm(int nx, int ny, int tc_mode) {
   return nx == 2048 ? iterate_kernel_slm_lx<11>(log2_exact(ny)) : nullptr;
 }
 
-// threads per block of the kernel of an nx x ny grid (not the general kernel,
-// whose block depends on the run)
+// threads per block of the kernel of an nx x ny grid (the general kernel's
+// block depends on the run: here its smallest one, kGenMinGeom)
 static int iteration_threads(int nx, int ny, int tc_mode) {
   return (uses_general(nx, ny) || tc_mode != kTcNone) ? kThreads : kThreads * iteration_split(nx, ny);
 }
@@ -149,7 +149,7 @@ static int mixed_threads(int tc_mode) { return tc_mode != kTcNone ? kThreads : k
 
 size_t iteration_smem_bytes(int nx, int ny, int tc_mode) {
   if (uses_rg(nx, ny)) return rg_smem_bytes(nx, ny);
-  if (uses_general(nx, ny)) return gen_smem_bytes(nx, ny, 4);
+  if (uses_general(nx, ny)) return gen_smem_bytes(nx, ny, kGenMinGeom.teams);
   // group exchange buffers, one column block of the amplitude, one of the
   // field; then the split-exchange buffers, or the tensor-core tables (and,
   // for tcgen05, operands)

@@ -134,3 +134,30 @@ def test_loss_rejects_general_grids():
         assert B.gs_physical_error(h, x.data_ptr(), x.data_ptr(), out.data_ptr()) == GS_EINVAL
     finally:
         B.gs_destroy(h)
+
+
+@pytest.mark.parametrize("ny,nx", [(480, 640), (90, 120), (9, 1536)])
+def test_fixed_grids_of_several_blocks_per_sm(ny, nx):
+    """gs_set_grid is clamped to what the device keeps resident, which on these
+    sides is more than one block of the general kernel per SM; the masks do not
+    depend on it."""
+    import torch
+
+    from paper_1302_0120_gb300 import GerchbergSaxton, build_lib
+    from paper_1302_0120_gb300 import _binding as B
+
+    build_lib.build()
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    I = torch.from_numpy(np.random.default_rng(5).random((ny, nx), dtype=np.float32)).cuda()
+    P = torch.from_numpy(S.random_phase(6, ny, nx)).cuda()
+    with GerchbergSaxton(nx, ny) as gs:
+        ref, _, _ = gs.run(I, P, 4)
+        for ctas in (sms - 1, sms + 20, 100000):
+            gs.set_grid(ctas)
+            assert B.gs_set_trace(gs.handle, True) == 0
+            ph, _, _ = gs.run(I, P, 4)
+            assert gs.status() == 0
+            assert torch.equal(ph, ref)
+            assert B.gs_get_trace(gs.handle).shape[1] == gs.grid
+            assert gs.grid == ctas or (ctas == 100000 and gs.grid > sms), gs.grid
+        assert B.gs_check_workspace(gs.handle) == B.GS_OK
