@@ -354,9 +354,11 @@ int gs_set_grid(gs_ctx* c, int ctas);
 int gs_test_barrier_timeout(gs_ctx* c, int enable);
 
 /*
- * gs_get_grid -- the number of thread blocks of the persistent kernel for a
- * run of one mask. A batch may take more of them, and a run on the small-grid
- * kernel (see gs_run) takes its clusters instead.
+ * gs_get_grid -- the number of thread blocks the next run will launch, if it
+ * has as many masks as the context was created for (max_batch; of every size,
+ * for a mixed context). A run of fewer masks may launch fewer; a run on the
+ * small-grid kernel (see gs_run) launches its clusters instead, and the number
+ * is that of the persistent kernel for it.
  * Writes it to *ctas (host). Returns GS_EINVAL for NULL arguments.
  */
 int gs_get_grid(gs_ctx* c, int* ctas);

@@ -328,6 +328,18 @@ int choose_grid(const gs_ctx* c, int masks) {
   return choose_grid_for(c, static_cast<long long>(c->nx) * c->ny * masks);
 }
 
+// Blocks of a mixed run of batch[k] masks of 256 << k: the single-size rule for
+// the class with the most pixels in a mask group.
+int choose_mixed_grid(const gs_ctx* c, const int* batch) {
+  long long px = 0;
+  for (int k = 0; k < 3; ++k) {
+    const long long n = static_cast<long long>(256 << k) * (256 << k);
+    const long long in_group = batch[k] > 0 ? n * group_size(c, n, batch[k]) : 0;
+    if (in_group > px) px = in_group;
+  }
+  return choose_grid_for(c, px);
+}
+
 }  // namespace
 
 namespace gsk {
@@ -608,14 +620,7 @@ int gs_run_mixed(gs_ctx* c, const int* batch, const float* const* target_intensi
     total += batch[k];
   }
   if (total < 1) return GS_EINVAL;
-  // the single-size rule for the class with the most pixels in a mask group
-  long long px = 0;
-  for (int k = 0; k < 3; ++k) {
-    const long long n = static_cast<long long>(256 << k) * (256 << k);
-    const long long in_group = batch[k] > 0 ? n * group_size(c, n, batch[k]) : 0;
-    if (in_group > px) px = in_group;
-  }
-  const int grid = choose_grid_for(c, px);
+  const int grid = choose_mixed_grid(c, batch);
   const Layout& P = c->L;  // the primary class holds the barrier, status and abort words
   unsigned char* const pw = c->ws;
   gsk::MixedParams mp{};
@@ -949,14 +954,8 @@ int gs_set_grid(gs_ctx* c, int ctas) {
 
 int gs_get_grid(gs_ctx* c, int* ctas) {
   if (c == nullptr || ctas == nullptr) return GS_EINVAL;
-  if (c->mixed) {
-    int largest = 0;
-    for (int k = 0; k < 3; ++k)
-      if (c->mixed_max[k] > 0) largest = k;
-    *ctas = choose_grid_for(c, static_cast<long long>(256 << largest) * (256 << largest));
-    return GS_OK;
-  }
-  *ctas = choose_grid(c, 1);
+  *ctas = c->mixed ? choose_mixed_grid(c, c->mixed_max)
+                   : choose_grid(c, group_size(c, static_cast<long long>(c->nx) * c->ny, c->max_batch));
   return GS_OK;
 }
 

@@ -97,3 +97,40 @@ def test_batch_with_an_invalid_target_across_launches():
     assert np.all(ph[0] == 9.0) and np.all(np.isnan(r[0]))
     ph1, r1, _, _ = gpu_gs(I[1], P[1], 140)
     assert np.array_equal(ph[1], ph1) and same_gaps(r[1], r1)
+
+
+@pytest.mark.parametrize("ny,nx,masks,group", [(512, 512, 4, 0), (256, 256, 16, 0), (256, 256, 16, 2), (1024, 1024, 2, 0),
+                                               (90, 120, 4, 0), (600, 800, 3, 1)])
+def test_reported_grid_is_launched(ny, nx, masks, group):
+    """gs_get_grid answers with the blocks that a full batch launches, also for
+    mask groups, where a batch takes more blocks than one of its masks."""
+    import torch
+
+    from paper_1302_0120_gb300 import GerchbergSaxton, build_lib
+    from paper_1302_0120_gb300 import _binding as B
+
+    build_lib.build()
+    I, P = (torch.from_numpy(x).cuda() for x in make_batch(masks, ny, nx, nspots=4))
+    with GerchbergSaxton(nx, ny, max_batch=masks) as gs:
+        gs.set_mask_group(group)
+        assert B.gs_set_trace(gs.handle, True) == 0
+        gs.run_batched(I, P, 2)
+        assert gs.status() == 0
+        assert B.gs_get_trace(gs.handle).shape[1] == gs.grid
+
+
+@pytest.mark.parametrize("counts", [{256: 64}, {256: 2, 512: 1}, {256: 8, 1024: 1}, {512: 16}])
+def test_reported_grid_of_a_mixed_context(counts):
+    """A mixed launch takes the grid of its class with the most pixels."""
+    from paper_1302_0120_gb300 import GerchbergSaxton, MixedGerchbergSaxton, build_lib
+
+    build_lib.build()
+    with MixedGerchbergSaxton(counts) as gm:
+        mixed = gm.grid
+    single = []
+    for n, k in counts.items():
+        with GerchbergSaxton(n, n, max_batch=k) as gs:
+            single.append(gs.grid)
+    assert mixed == max(single)
+    n, k = max(counts.items(), key=lambda e: e[0] * e[0] * e[1])
+    assert mixed >= min(152, n * n * k // 4096)
