@@ -7,13 +7,17 @@ namespace gsk {
 
 // sum p^2 in FP64, in a fixed order; NaN if any p is negative or not finite.
 // Each block a contiguous share into scratch, eight loads of a thread in
-// flight; then one warp adds the blocks. (One block for all of it took 580 us
-// at 1024 x 1024, now 6.)
+// flight; then one warp adds the blocks. Up to 4096 values are one block, which
+// writes the sum itself. Microseconds a call with one block of 1024 threads and
+// a load at a time for everything, with two launches for everything, and now:
+// 8 x 8 6.2, 8.3, 4.2; 64 x 64 8.3, 10.3, 6.3; 128 x 128 14.5, 10.3, 10.3; 1024 x
+// 1024 577, 12.5, 12.5. (One block of 1024 threads up to 128 x 128: 10.4 at 64 x
+// 64 and 14.5 at 128 x 128, the FP64 pipe of one SM.)
 constexpr int kEnergyThreads = 256;
 constexpr int kEnergyBlocks = kMaxGrid;
 
 __global__ void __launch_bounds__(kEnergyThreads) energy_kernel(const float* __restrict__ p, long long n,
-                                                               double* __restrict__ scratch) {
+                                                               double* __restrict__ to) {
   __shared__ double red[kEnergyThreads / 32];
   const long long lo = blockIdx.x * n / gridDim.x, hi = (blockIdx.x + 1) * n / gridDim.x;
   double acc = 0.0;
@@ -35,7 +39,7 @@ __global__ void __launch_bounds__(kEnergyThreads) energy_kernel(const float* __r
   if (threadIdx.x == 0) {
     double s = 0.0;
     for (int w = 0; w < kEnergyThreads / 32; ++w) s += red[w];
-    scratch[blockIdx.x] = any_bad ? __longlong_as_double(0x7ff8000000000000ll) : s;
+    to[blockIdx.x] = any_bad ? __longlong_as_double(0x7ff8000000000000ll) : s;
   }
 }
 
@@ -50,8 +54,8 @@ __global__ void __launch_bounds__(32) energy_total(const double* __restrict__ sc
 cudaError_t launch_energy(const float* p, long long n, double* energy, double* scratch, cudaStream_t s) {
   const long long want = (n + 4095) / 4096;
   const int blocks = static_cast<int>(want < kEnergyBlocks ? want : kEnergyBlocks);
-  energy_kernel<<<blocks, kEnergyThreads, 0, s>>>(p, n, scratch);
-  energy_total<<<1, 32, 0, s>>>(scratch, blocks, energy);
+  energy_kernel<<<blocks, kEnergyThreads, 0, s>>>(p, n, blocks == 1 ? energy : scratch);
+  if (blocks > 1) energy_total<<<1, 32, 0, s>>>(scratch, blocks, energy);
   return cudaGetLastError();
 }
 

@@ -83,3 +83,29 @@ def test_target_start(n, iters):
     tol = max(1e-5, 3 * aligned_rel_err(fp32["phase"].astype(np.float32), ref0["u"]))
     assert st == 0 and aligned_rel_err(ph0, ref0["u"]) <= tol
     assert abs(r0[0] - ref0["r"][0]) <= 1e-4 * ref0["r"][0]
+
+
+@pytest.mark.parametrize("ny,nx", [(8, 8), (9, 27), (64, 64), (40, 128), (128, 128), (1000, 1250)])
+def test_laser_energy(ny, nx):
+    """sum p^2 (by one block, or by several and their total) against FP64: r^0 of
+    p = c is that of p = 1 with its field and target scaled by c, and a bad
+    pixel anywhere, the last one included, is found."""
+    from paper_1302_0120_gb300 import GS_ENUMERIC
+
+    rng = np.random.default_rng(ny * nx)
+    I = rng.random((ny, nx), dtype=np.float32)
+    phi0 = S.random_phase(81, ny, nx)
+    p = (0.25 + rng.random((ny, nx), dtype=np.float32)).astype(np.float32)
+    _, r, g, st = gpu_run(I, phi0, 1, p=p)
+    assert st == 0
+    # r^0 is a ratio to sqrt(sum p^2), with a target scaled by it: FP32 fields
+    # against FP64 (as in test_laser_amplitude), the energy itself in FP64
+    e = float(np.sum(p.astype(np.float64) ** 2))
+    u = p.astype(np.float64) * np.exp(1j * phi0.astype(np.float64))
+    _, r0, g0 = O.gs_step(u, O.target_amplitude(I, energy=e), p.astype(np.float64))
+    assert abs(r[0] - r0) <= 1e-5 * r0 and abs(g[0] - g0) <= 1e-5 * g0
+    for at in (0, p.size - 1):
+        bad = p.copy()
+        bad.flat[at] = np.nan
+        _, r, _, st = gpu_run(I, phi0, 1, p=bad)
+        assert st == GS_ENUMERIC and np.all(np.isnan(r))
