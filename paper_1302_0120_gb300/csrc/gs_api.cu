@@ -71,7 +71,7 @@ constexpr int kTwiddleEntries = gsk::kStageTwiddleEntries;
 
 // Offsets of the sub-buffers of one workspace allocation.
 struct Layout {
-  size_t B, mT, partials, twx, twy, ones, bar, status, abort_flag, mask_flags, energy, lossbuf, dI, dphi, trace, total;
+  size_t B, mT, partials, twx, twy, bar, status, abort_flag, mask_flags, energy, lossbuf, dI, dphi, trace, total;
   size_t guard[16];  // canary words after each buffer (gs_check_workspace)
   int nguard;
 };
@@ -94,8 +94,6 @@ Layout make_layout(int nx, int ny, int max_batch) {
   L.twx = o;        o = align_up(o + static_cast<size_t>(kTwiddleEntries) * sizeof(float2));
   L.guard[L.nguard++] = o; o += kGuardBytes;
   L.twy = o;        o = align_up(o + static_cast<size_t>(kTwiddleEntries) * sizeof(float2));
-  L.guard[L.nguard++] = o; o += kGuardBytes;
-  L.ones = o;       o = align_up(o + 4096 * sizeof(float));
   L.guard[L.nguard++] = o; o += kGuardBytes;
   // the barrier counter and the abort word side by side: one memset clears
   // both before the first launch of a run
@@ -417,9 +415,7 @@ int gs_create_batched(gs_ctx** out, int nx, int ny, int max_batch, unsigned flag
   const bool rg = gsk::uses_rg(nx, ny);
   const std::vector<float2> wx = rg ? rg_twiddles(nx) : twiddles(nx, general);
   const std::vector<float2> wy = rg ? rg_twiddles(ny) : twiddles(ny, general);
-  const std::vector<float> ones(4096, 1.0f);
   bool ok = cudaMemcpy(c->ws + c->L.twx, wx.data(), wx.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
-            cudaMemcpy(c->ws + c->L.ones, ones.data(), ones.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemcpy(c->ws + c->L.twy, wy.data(), wy.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaMemset(c->ws + c->L.bar, 0, c->L.dI - c->L.bar) == cudaSuccess && fill_guards(c->ws, c->L);
   if (!ok) {
@@ -485,7 +481,6 @@ int gs_run_batched(gs_ctx* c, int batch, const float* target_intensity, const fl
   p.mask_flags = at<int>(c, c->L.mask_flags);
   p.p_slm = c->p_slm;
   p.energy = at<double>(c, c->L.energy);
-  p.ones = at<float>(c, c->L.ones);
   p.init_target = from_target ? 1 : 0;
   p.iters = iters;
   p.final_resid = (c->flags & GS_FINAL_RESIDUAL) ? 1 : 0;
@@ -652,7 +647,6 @@ int gs_run_mixed(gs_ctx* c, const int* batch, const float* const* target_intensi
     p.partials = reinterpret_cast<double*>(w + L.partials);
     p.twx = reinterpret_cast<const float2*>(w + L.twx);
     p.twy = reinterpret_cast<const float2*>(w + L.twy);
-    p.ones = reinterpret_cast<const float*>(w + L.ones);
     p.mask_flags = reinterpret_cast<int*>(w + L.mask_flags);
     p.energy = reinterpret_cast<const double*>(w + L.energy);
     if (batch[k] == 0) continue;

@@ -113,46 +113,29 @@ __device__ __forceinline__ int small_div(int a, int b) {
 template <int R>
 __device__ __forceinline__ void gen_stage(const float2* __restrict__ src, float2* __restrict__ dst, int n, int ns,
                                           const float2* __restrict__ tw, const GenTeam& tm) {
-  constexpr int U = 1;
   const int nb = n / R;
   const int tt = tm.t;
   const int qinc = small_div(tm.T, ns), rinc = tm.T - qinc * ns;
   int q = small_div(tt, ns), r = tt - q * ns;
   const float2* const tws = tw + (ns - 1);
-  for (int j0 = tt; j0 < nb; j0 += tm.T * U) {
-    float2 a[U][R];
-    int base[U], rr[U];
+  for (int j = tt; j < nb; j += tm.T) {
+    float2 a[R];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int j = j0 + tm.T * u;
-      rr[u] = r;
-      base[u] = q * ns * R + r;
-      if (j < nb) {
-#pragma unroll
-        for (int m = 0; m < R; ++m) a[u][m] = src[j + m * nb];
-      }
-      q += qinc;
-      r += rinc;
-      if (r >= ns) {
-        r -= ns;
-        ++q;
-      }
-    }
+    for (int m = 0; m < R; ++m) a[m] = src[j + m * nb];
     if (ns > 1) {
 #pragma unroll
-      for (int u = 0; u < U; ++u)
-        if (j0 + tm.T * u < nb) {
-#pragma unroll
-          for (int m = 1; m < R; ++m) a[u][m] = cmul(a[u][m], tws[(m - 1) * ns + rr[u]]);
-        }
+      for (int m = 1; m < R; ++m) a[m] = cmul(a[m], tws[(m - 1) * ns + r]);
     }
+    small_dft<R>(a);
+    float2* const to = dst + q * ns * R + r;
 #pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (j0 + tm.T * u < nb) {
-        small_dft<R>(a[u]);
-#pragma unroll
-        for (int k = 0; k < R; ++k) dst[base[u] + k * ns] = a[u][k];
-      }
+    for (int k = 0; k < R; ++k) to[k * ns] = a[k];
+    q += qinc;
+    r += rinc;
+    if (r >= ns) {
+      r -= ns;
+      ++q;
+    }
   }
 }
 

@@ -69,7 +69,6 @@ struct Params {
   int final_resid;     // compute r^K
   const float* p_slm;  // SLM amplitude p [ny][nx] (Eq. slm-constraint), or null for p = 1
   const double* energy;  // sum p^2 (FP64, workspace) when p_slm is set
-  const float* ones;   // a row of max(nx, ny) ones (workspace): p when p_slm is null
   int init_target;     // start from P_S(F^{-1} m) instead of p exp(i phi_in)
   unsigned extra_arrivals;  // test hook: arrivals a barrier waits for beyond the grid (0 in use)
   float inv_sqrt_n;    // 1/sqrt(N)

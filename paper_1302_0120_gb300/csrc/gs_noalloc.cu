@@ -30,8 +30,7 @@ constexpr size_t kOffM = align_up(kOffB + static_cast<size_t>(kMaxPixels) * 8);
 constexpr size_t kOffPartials = align_up(kOffM + static_cast<size_t>(kMaxPixels) * 4);
 constexpr size_t kOffTwx = align_up(kOffPartials + static_cast<size_t>(gsk::kSlots) * kMaxGrid * 8);
 constexpr size_t kOffTwy = align_up(kOffTwx + static_cast<size_t>(kTwEntries) * 8);
-constexpr size_t kOffOnes = align_up(kOffTwy + static_cast<size_t>(kTwEntries) * 8);
-constexpr size_t kOffWords = align_up(kOffOnes + 4096 * sizeof(float));
+constexpr size_t kOffWords = align_up(kOffTwy + static_cast<size_t>(kTwEntries) * 8);
 constexpr size_t kScratchBytes = align_up(kOffWords + (3 + gsk::kMaxBatch) * sizeof(int));  // barrier, status, abort, mask flags
 
 // The shared scratch of every gs_run_noalloc call on this device (about 4 MiB).
@@ -83,10 +82,6 @@ __global__ void twiddle_tables(float2* tw, int n) {
     }
     tw[e] = w;
   }
-}
-
-__global__ void fill_ones(float* x, int n) {
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n; e += gridDim.x * blockDim.x) x[e] = 1.0f;
 }
 
 // Device address of the static scratch on the current device; looked up on
@@ -162,7 +157,6 @@ extern "C" int gs_run_noalloc(int nx, int ny, unsigned flags, void* stream, cons
   p.status = reinterpret_cast<int*>(base + kOffWords) + 1;
   p.abort_flag = reinterpret_cast<int*>(base + kOffWords) + 2;
   p.mask_flags = reinterpret_cast<int*>(base + kOffWords) + 3;
-  p.ones = reinterpret_cast<const float*>(base + kOffOnes);
   p.batch = 1;
   p.group = 1;
   p.init_target = from_target ? 1 : 0;
@@ -182,7 +176,6 @@ extern "C" int gs_run_noalloc(int nx, int ny, unsigned flags, void* stream, cons
     cudaGetLastError();
     return GS_ECUDA;
   }
-  fill_ones<<<16, 256, 0, s>>>(reinterpret_cast<float*>(base + kOffOnes), 4096);
   twiddle_tables<<<64, 256, 0, s>>>(const_cast<float2*>(p.twx), nx);
   twiddle_tables<<<64, 256, 0, s>>>(const_cast<float2*>(p.twy), ny);
   if (cudaGetLastError() != cudaSuccess) return GS_ECUDA;

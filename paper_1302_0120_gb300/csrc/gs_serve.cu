@@ -104,7 +104,6 @@ int gs_serve_create(gs_server** out, int max_n, int slots, int grid, void* strea
   const size_t omT = o;   o = align_up(o + slots * npix * sizeof(float));
   const size_t opart = o; o = align_up(o + 3 * static_cast<size_t>(kServeMaxSlots) * s->grid * sizeof(double));
   const size_t otw = o;   o = align_up(o + 3 * static_cast<size_t>(gsk::kStageTwiddleEntries) * sizeof(float2));
-  const size_t oones = o; o = align_up(o + 4096 * sizeof(float));
   const size_t obar = o;  o = align_up(o + sizeof(unsigned));
   const size_t ostat = o; o = align_up(o + sizeof(int));
   const size_t oabort = o; o = align_up(o + sizeof(int));
@@ -112,7 +111,6 @@ int gs_serve_create(gs_server** out, int max_n, int slots, int grid, void* strea
   const size_t ost = o;   o = align_up(o + sizeof(gsk::ServeState));
   std::vector<float2> tw(3 * static_cast<size_t>(gsk::kStageTwiddleEntries));
   for (int k = 0; 8 + k <= L; ++k) gsk::stage_twiddles_host(256 << k, tw.data() + k * gsk::kStageTwiddleEntries);
-  const std::vector<float> ones(4096, 1.0f);
   if (cudaMalloc(&s->ws, o) != cudaSuccess) {
     cudaGetLastError();
     delete s;
@@ -129,7 +127,6 @@ int gs_serve_create(gs_server** out, int max_n, int slots, int grid, void* strea
   bool ok = cudaHostGetDevicePointer(reinterpret_cast<void**>(&dtab), s->table, 0) == cudaSuccess &&
             cudaMemset(s->ws, 0, o) == cudaSuccess &&
             cudaMemcpy(s->ws + otw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice) == cudaSuccess &&
-            cudaMemcpy(s->ws + oones, ones.data(), ones.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess &&
             cudaEventCreateWithFlags(&s->ev, cudaEventDisableTiming) == cudaSuccess;
   if (!ok) {
     cudaGetLastError();
@@ -149,7 +146,6 @@ int gs_serve_create(gs_server** out, int max_n, int slots, int grid, void* strea
     s->sp.tw[k] = 8 + k <= L ? reinterpret_cast<const float2*>(s->ws + otw) + k * gsk::kStageTwiddleEntries : nullptr;
   s->sp.max_log = L;
   s->sp.max_ticks = gsk::kServeMaxTicks;
-  p.ones = reinterpret_cast<const float*>(s->ws + oones);
   p.bar = reinterpret_cast<unsigned*>(s->ws + obar);
   p.status = reinterpret_cast<int*>(s->ws + ostat);
   p.abort_flag = reinterpret_cast<int*>(s->ws + oabort);
