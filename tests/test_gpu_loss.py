@@ -459,3 +459,34 @@ def test_nonfinite_target():
     I[3, 3] = np.inf
     loss, grad, st = gpu_loss_grad(I, S.random_phase(2, 64, 64))
     assert st == GS_ENUMERIC and np.isnan(loss)
+
+
+# The lengths between and beyond the oracle's: 128 and 512 (early end of the row
+# passes), 2048 and 4096 (three stages, teams of 64 and 128 lanes on named
+# barriers). FP64 reference by torch.fft. An FP32 transform of n^2 points has a
+# relative error of some eps log2(n^2) / 2 (7e-7 at 4096), the gradient two of
+# them; the sums add a few eps. Gate 1e-5.
+@pytest.mark.parametrize("n", [128, 512, 2048, 4096])
+def test_loss_and_gradient_match_fp64_fft(n):
+    import torch
+
+    I = normalized_target(n + 2, n, 40)
+    phi = S.random_phase(n + 3, n, n)
+    loss, grad, st = gpu_loss_grad(I, phi)
+    assert st == 0
+    I64, phi64 = (torch.from_numpy(x).cuda().double() for x in (I, phi))
+    x = torch.polar(torch.ones_like(phi64), phi64)
+    y = torch.fft.fft2(x)
+    r = y.abs() ** 2 / (n * n) - I64
+    ref_l = float((r * r).sum())
+    ref_g = 4 * (x.conj() * torch.fft.ifft2(r * y)).imag
+    assert abs(loss - ref_l) <= 1e-5 * ref_l, (loss, ref_l)
+    err = torch.linalg.norm(torch.from_numpy(grad).cuda().double() - ref_g) / torch.linalg.norm(ref_g)
+    assert float(err) <= 1e-5, float(err)
+    loss_only, none, st = gpu_loss_grad(I, phi, want_grad=False)
+    assert st == 0 and none is None and loss_only == loss
+
+
+@pytest.mark.parametrize("n,steps", [(32, 3), (128, 5), (512, 12), (2048, 3), (4096, 2)])
+def test_fused_run_matches_single_launches_at_other_lengths(n, steps):
+    test_fused_run_matches_single_launches(n, steps)

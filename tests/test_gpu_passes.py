@@ -165,3 +165,55 @@ def test_laser_step_on_long_rows(ny, nx):
     b = torch.polar(p64, torch.angle(v))
     c = (a.conj() * b).sum()
     assert float(torch.linalg.norm(a * (c / c.abs()) - b) / torch.linalg.norm(b)) <= 1e-5
+
+
+# The target start: a column pass that transforms the amplitude itself, without
+# copies ahead, then a row pass, each in several rounds on a small grid.
+@pytest.mark.parametrize("ny,nx,grid", [(256, 256, 3), (512, 512, 7), (1024, 1024, 9), (2048, 1024, 23), (600, 800, 11),
+                                        (480, 640, 9)])
+def test_target_start_rounds_match_one_round(ny, nx, grid):
+    import torch
+
+    from paper_1302_0120_gb300 import GerchbergSaxton, build_lib
+
+    build_lib.build()
+    I = torch.from_numpy(S.spot_target(75, ny, nx, 9, (0.5, 1.0))).cuda()
+    out = []
+    for g in (0, grid):
+        with GerchbergSaxton(nx, ny, init_from_target=True) as gs:
+            gs.set_grid(g)
+            res = gs.run(I, None, 3)
+            out.append(tuple(x.cpu().numpy() for x in res) + (gs.status(),))
+    _same(*out)
+
+
+# |z|^2 below the smallest normal number takes the long form of the projections.
+# A laser amplitude of a power of two 2^-k everywhere scales every field of the
+# run by it and changes no mask, but for the rounding of subnormal |z|^2: an
+# error of 2^-150 in |z|^2, which is exponentially distributed about 2^-122 here
+# (6 % of it below 2^-126, in nearly every thread), is one of
+# 2^-150 sqrt(N) / 2^-121 (2e-6 at 1024^2) in the root mean square of a field.
+@pytest.mark.parametrize("ny,nx", [(64, 64), (256, 256), (1024, 1024), (600, 800), (480, 640)])
+def test_subnormal_fields_give_the_same_mask(ny, nx):
+    k = round((122 + np.log2(ny * nx)) / 2)  # |z|^2 about N 4^-k
+    I = S.spot_target(76, ny, nx, 9, (0.5, 1.0))
+    phi0 = S.random_phase(77, ny, nx)
+    one = _laser_run(I, phi0, np.ones((ny, nx), np.float32), 1)
+    tiny = _laser_run(I, phi0, np.full((ny, nx), 2.0 ** -k, np.float32), 1)
+    assert one[3] == 0 and tiny[3] == 0
+    assert aligned_rel_err(tiny[0], np.exp(1j * one[0].astype(np.float64))) <= 1e-5
+    # the gaps: terms of some 4^-k, rounded to 2^-149 where they are subnormal
+    np.testing.assert_allclose(tiny[1], one[1], rtol=1e-3)
+    np.testing.assert_allclose(tiny[2], one[2], rtol=1e-3)
+
+
+# Sides up to 4096 beside short ones: as long as the lines fit shared memory.
+@pytest.mark.parametrize("ny,nx", [(100, 2048), (2048, 100), (320, 320), (50, 600)])
+def test_general_long_sides_parity(ny, nx):
+    I = S.spot_target(78, ny, nx, 6, (0.5, 1.0))
+    phi0 = S.random_phase(79, ny, nx)
+    ph, r, g, st = gpu_gs(I, phi0, 1)
+    assert st == 0
+    u, r0, g0 = O.gs_step(np.exp(1j * phi0.astype(np.float64)), O.target_amplitude(I))
+    assert aligned_rel_err(ph, u) <= 1e-5
+    assert abs(r[0] - r0) <= 1e-5 * r0 and abs(g[0] - g0) <= 1e-5 * g0
