@@ -30,7 +30,10 @@
  *     (2^a 3^b 5^c, such as the 800 x 600 SLM of Sec. V) in [8, 1536].
  *     Grids with both sides powers of two of at least 32 run on the
  *     register-resident kernels (one cluster per mask when the grid has at
- *     most 32768 pixels, see gs_run); every other grid on the general kernel.
+ *     most 32768 pixels, see gs_run); every other grid on the general kernel,
+ *     whose lines a block keeps in shared memory: for a side of 4096 beside one
+ *     that is not a power of two or is below 32 there is no room, and
+ *     gs_create returns GS_ECUDA.
  *
  * Memory and ordering:
  *   - Pointers named "device" are CUDA device pointers owned by the caller;
@@ -170,8 +173,8 @@ int gs_run(gs_ctx* c, const float* target_intensity, const float* phase_in, int 
  *
  * Operation: Eq. (e:AP) for each mask b < batch, exactly as gs_run (the
  * masks share only the launch: phases are identical to separate runs; the
- * gaps agree to FP64 rounding, their partial sums being grouped by the
- * blocks' shares of the whole batch).
+ * gaps agree to the rounding of a block's FP32 partial sum, about 1e-6, the
+ * sums being grouped by the blocks' shares of the whole batch).
  * Every array is strided by mask, mask b at offset b * (per-mask size):
  *   target_intensity, phase_in, phase_out  device, float [batch][ny][nx]
  *   residual_out   device, double [batch][K+1] (GS_FINAL_RESIDUAL) or
@@ -208,11 +211,12 @@ int gs_create_mixed(gs_ctx** out, const int* max_batch, unsigned flags, void* st
  * size n_k = 256 << k (k = 0, 1, 2) in one persistent launch (chunks of 128
  * iterations, as gs_run).
  *
- * Every pass of the launch visits the masks of all three sizes before its
- * grid barrier; each mask follows exactly the single-size path (same
- * transforms, projections and gaps), so its phase is bit-identical to a
- * gs_run_batched run of its size; its gaps can differ in the last bits
- * because the FP64 partial sums are grouped by the launch's block count.
+ * The sizes run one after the other, each (in mask groups) through the
+ * schedule of passes of the launch; each mask follows exactly the single-size
+ * path (same transforms, projections and gaps), so its phase is bit-identical
+ * to a gs_run_batched run of its size; its gaps can differ by about 1e-6, the
+ * rounding of a block's FP32 partial sum, because these are grouped by the
+ * launch's block count.
  *   batch            host int[3], 0 <= batch[k] <= max_batch[k], sum >= 1.
  *   target_intensity host array of 3 device pointers; entry k: float
  *                    [batch[k]][n_k][n_k] (ignored when batch[k] = 0).
@@ -323,7 +327,7 @@ int gs_get_trace(gs_ctx* c, unsigned long long* host_out, int capacity, int* pas
  * A batch runs group after group, each group through the whole iteration
  * schedule of the launch, so that a group's fields (12 bytes per pixel) can
  * stay in L2; results do not depend on it (phases bit-identical, gaps to
- * FP64 rounding). masks = 0 (the default) takes, per grid size, the most
+ * about 1e-6, the rounding of a block's FP32 partial sum). masks = 0 (the default) takes, per grid size, the most
  * masks whose fields fit 100 MiB (8 of 1024 x 1024); masks > 0 fixes the
  * group size, capped by the batch. In a mixed run the sizes always run one
  * after the other. Returns GS_EINVAL for a NULL context or masks < 0.

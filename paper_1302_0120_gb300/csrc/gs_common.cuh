@@ -70,7 +70,9 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // Added once to the grid-barrier counter by the first failing thread of a
 // launch: it releases every waiting block, which sees the bit in the value its
 // spin ended on (no extra load after the barrier). Arrivals per launch stay far
-// below it (at most blocks x passes, < 2^20).
+// below it: one per block and barrier, and every mask group of a launch runs
+// the whole schedule of at most kSlots + 4 barriers (256 blocks, 64 groups:
+// 2^22.1; of a mixed launch, whose masks are 64 in all, no more).
 constexpr unsigned kAbortBit = 1u << 30;
 
 __device__ __forceinline__ void fail(const Params& p, int code) {

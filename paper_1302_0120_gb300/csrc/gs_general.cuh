@@ -1,6 +1,6 @@
 // gs_general.cuh -- passes of the iteration kernel for grids whose sides are
-// not powers of two (any 5-smooth side 2^a 3^b 5^c in [32, 1536]), such as
-// the 800 x 600 SLM of Sec. V.
+// not powers of two or are below 32 (5-smooth sides 2^a 3^b 5^c in [8, 1536],
+// also beside a power of two up to 2048), except those of gs_rg.cuh.
 //
 // The pass structure, projections and FP64 gap sums are those of the
 // power-of-two kernel (gs_iterate.cuh); what differs is the transform and the
@@ -20,9 +20,8 @@
 //     each team transforms, projects and transforms its column, and the block
 //     writes the tile back the same way.
 //   * A length-n transform is a Stockham auto-sort FFT with radices 3 and 5
-//     first, then 8, 4 and 2 (gen_fft), each stage read from one of the warp's
-//     two buffers and written to the other. The
-//     twiddles of the stage with sub-transform length ns and radix R sit at
+//     first, then 8, 4 and 2 (gen_fft), each stage read from one of the team's
+//     two buffers and written to the other. The twiddles of the stage with sub-transform length ns and radix R sit at
 //     entries ns - 1 + (m - 1) ns + r (W_{ns R}^{r m}), so that consecutive
 //     butterflies read consecutive entries; the tables are rounded once from
 //     double on the host and copied to shared memory per launch.
@@ -206,7 +205,7 @@ __device__ __forceinline__ float gen_phase(float2 u) {
 }
 
 // One pass over rows [lo, hi) (kInit, kRow) or columns [lo, hi)
-// (kCol, kResid, kInitM) of mask mb. Returns this thread's FP64 contribution
+// (kCol, kResid, kInitM) of mask mb. Returns this thread's FP32 contribution
 // to the pass's gap sum.
 static __device__ __forceinline__ float run_pass_gen(const Params& p, int mb, int kind, bool last, int lo, int hi,
                                                       unsigned char* smem) {
@@ -302,7 +301,7 @@ static __device__ __forceinline__ float run_pass_gen(const Params& p, int mb, in
   // Column passes: groups of adjacent columns; team k owns column c0 + k.
   const int stride = gen_team_stride(nmax);
   const bool store = (kind == kCol || kind == kInitM);
-  // which of a warp's buffers holds the stored result: A after two transforms,
+  // which of a team's buffers holds the stored result: A after two transforms,
   // else A or Bf by the parity of the stage count
   const int out_off = (kind == kCol || (p.nsty & 1) == 0) ? 0 : nmax + 1;
   // the tile's copies: this thread's column of the group, and its first row

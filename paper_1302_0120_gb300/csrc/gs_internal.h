@@ -264,7 +264,7 @@ struct LossParams {
   double* phys;            // [2]: physical error (E_l, E_d), or null
   const float* p_slm;      // SLM amplitude [n][n], or null (p = 1)
   const double* energy;    // sum p^2 when p_slm is set
-  double* partials;        // [6][grid]
+  double* partials;        // rows of LossRow (gs_loss.cuh): six of `grid` values, three of kMaxGrid
   const float2* tw;        // stage twiddle tables (length n)
   unsigned* bar;
   int* status;

@@ -28,8 +28,8 @@
 // real and imaginary parts, which is folded into the projections, so B holds
 // swap(IDFT_y(Yhat)) between a column pass and the next row pass.
 //
-// FP64 is used only for the per-block partial sums of the target energy and
-// of the two gaps; the field is FP32.
+// FP64 is used only for the sums of the target energy and, across blocks, of the
+// two gaps (FP32 within a block); the field is FP32.
 #pragma once
 
 #include <cfloat>

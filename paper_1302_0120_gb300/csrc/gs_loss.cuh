@@ -463,9 +463,12 @@ __global__ void __launch_bounds__(kThreads * kLossSplit, 1) gs_loss_kernel(const
       const int hi = split(b + 1, gridDim.x, N);
       const float scale = 4.f * p.inv_n;
       for (int base = lo; base < hi; base += NG) {
-        // no row for this team (half of the teams at 512 x 512: 1.86 -> 1.68 ms
-        // per 100 steps; at 1024 x 1024 and above few are idle, and the loop
-        // that may end early was slower: 4.26 -> 4.57 ms per 200)
+        // No row for this team. A block of the automatic grid has eight rows of
+        // 512 points for its 16 groups (of 256 points 8 for 32), so that half of
+        // the teams or more leave here: 1.86 -> 1.68 ms per 100 steps at 512 x
+        // 512. From 1024 points on it is one or two of eight (1024) or some in
+        // the last round, and the compiler's code for a loop that may end early
+        // lost more than that won (1024 x 1024 4.26 -> 4.57 ms per 200 steps).
         if (LN <= 9 && base + team_line >= hi) break;
         const int idx = base + gidx;
         const bool valid = idx < hi;

@@ -21,8 +21,9 @@ class GerchbergSaxton:
     def __init__(self, nx: int, ny: int, final_residual: bool = True, stream=None, max_batch: int = 1,
                  init_from_target: bool = False, tensor_core: bool = False, bf16: bool = False,
                  mma_sync: bool = False):
-        """``tensor_core`` runs the DFTs as FP16 tensor-core products (1024 x
-        1024 on tcgen05 unless ``mma_sync``; ``bf16`` for BF16 operands there)."""
+        """``tensor_core`` runs the DFTs as FP16 tensor-core products (square 256,
+        512 and 1024; on tcgen05 unless ``mma_sync``, ``bf16`` for split BF16
+        operands there)."""
         import torch
 
         if stream is None:
