@@ -660,7 +660,8 @@ __device__ __forceinline__ LateSum class_pass(const Params& p, Shared& sh, int b
     const int shi = min(hi, (mb - w0 + 1) * per) - (mb - w0) * per;
     float a;
     if constexpr (LX == 0) {
-      a = run_pass_gen(p, mb, f.kind, f.last, slo, shi, smem);
+      a = p.gen_team_log == 6 ? run_pass_gen<6>(p, mb, f.kind, f.last, slo, shi, smem)
+                              : run_pass_gen<7>(p, mb, f.kind, f.last, slo, shi, smem);
     } else if constexpr (is_rg_side(LX)) {
       a = run_pass_rg<LX, LY>(p, mb, f.kind, f.last, slo, shi, smem, sh, mphase);
     } else if constexpr (LX == LY) {
