@@ -297,6 +297,7 @@ int small_logc(const gs_ctx* c, int batch) {
 bool on_general(const gs_ctx* c) { return !c->mixed && gsk::uses_general(c->nx, c->ny) && !gsk::uses_rg(c->nx, c->ny); }
 
 // Blocks of a run on the general kernel, and their geometry.
+constexpr int kGenShortColumn = 40;  // points (gen_run)
 struct GenRun {
   gsk::GenGeom geom;
   int grid;
@@ -311,8 +312,23 @@ GenRun gen_run(const gs_ctx* c, int masks) {
     if (r.grid > c->num_sms) r.geom = gsk::kGenMinGeom;
     return r;
   }
-  // one block per SM at most, enough for one line per team and round
   const long long lines = static_cast<long long>(c->nx > c->ny ? c->nx : c->ny) * masks;
+  // Batches of short columns: a tile of them is hardly any work between the
+  // barriers of a block, and two of the smallest blocks on an SM fill each
+  // other's waits. They are taken where they need no more rounds, or a fifth
+  // more of many. Ten iterations with the large blocks and with the small ones
+  // (nx x ny, masks, microseconds): 512 x 16, 2 173 and 142; 1536 x 24, 4 376
+  // and 348; 1536 x 8, 64 2750 and 2382; 1500 x 20, 2 274 and 281 (the worst).
+  // With more rounds they lose (1500 x 20, 8 538 and 577) as often as they win.
+  const int cap = max_grid(c);
+  if (masks > 1 && c->ny <= kGenShortColumn && c->nx > c->ny && r.geom.team_log == gsk::kGenMinGeom.team_log &&
+      cap > c->num_sms) {
+    const long long small = static_cast<long long>(cap) * gsk::kGenMinGeom.teams;
+    const long long large = static_cast<long long>(c->num_sms) * r.geom.teams;
+    const long long rounds = (lines + large - 1) / large, more = (lines + small - 1) / small;
+    if (lines >= small && (more <= rounds || (rounds >= 8 && 5 * more <= 6 * rounds))) return {gsk::kGenMinGeom, cap};
+  }
+  // one block per SM at most, enough for one line per team and round
   const long long g = (lines + r.geom.teams - 1) / r.geom.teams;
   r.grid = static_cast<int>(g < c->num_sms ? g : c->num_sms);
   return r;

@@ -161,3 +161,33 @@ def test_fixed_grids_of_several_blocks_per_sm(ny, nx):
             assert B.gs_get_trace(gs.handle).shape[1] == gs.grid
             assert gs.grid == ctas or (ctas == 100000 and gs.grid > sms), gs.grid
         assert B.gs_check_workspace(gs.handle) == B.GS_OK
+
+
+@pytest.mark.parametrize("masks,ny,nx,laser", [(2, 16, 512, False), (4, 9, 1536, True), (16, 24, 1024, False),
+                                               (12, 40, 1200, True), (5, 8, 1500, False), (3, 40, 1536, False)])
+def test_batches_of_short_columns(masks, ny, nx, laser):
+    """Batches of long rows and short columns may take several small blocks per
+    SM: every mask of the batch equals its single run bit for bit, and the launch
+    has the grid that is reported."""
+    import torch
+
+    from paper_1302_0120_gb300 import GerchbergSaxton, build_lib
+    from paper_1302_0120_gb300 import _binding as B
+
+    build_lib.build()
+    rng = np.random.default_rng(nx + ny)
+    I = torch.from_numpy(rng.random((masks, ny, nx), dtype=np.float32)).cuda()
+    P = torch.from_numpy((2 * np.pi * rng.random((masks, ny, nx))).astype(np.float32)).cuda()
+    p = torch.from_numpy(S.laser_amplitude(ny, nx)).cuda() if laser else None
+    with GerchbergSaxton(nx, ny, max_batch=masks) as gs:
+        gs.set_slm_amplitude(p)
+        assert B.gs_set_trace(gs.handle, True) == 0
+        ph, r, g = gs.run_batched(I, P, 4)
+        assert gs.status() == 0 and B.gs_check_workspace(gs.handle) == B.GS_OK
+        assert B.gs_get_trace(gs.handle).shape[1] == gs.grid
+        for k in range(masks):
+            ph1, r1, g1 = gs.run(I[k], P[k], 4)
+            assert gs.status() == 0
+            assert torch.equal(ph[k], ph1)
+            np.testing.assert_allclose(r[k].cpu(), r1.cpu(), rtol=GROUPING_RTOL, atol=0)
+            np.testing.assert_allclose(g[k].cpu(), g1.cpu(), rtol=GROUPING_RTOL, atol=0)
